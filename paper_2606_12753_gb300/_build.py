@@ -23,7 +23,8 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INC
 # root use the hardware approximations (about 2 ulp instead of IEEE
 # rounding), well inside the 1e-5 tolerance of these forms.  FP64 divide and
 # square root are unaffected by these flags.
-FAST_FP32_UNITS = {"stage_mixed.cu", "stage_fp32.cu", "batch_mixed.cu", "batch_fp32.cu"}
+FAST_FP32_UNITS = {"stage_mixed.cu", "stage_fp32.cu", "stage2d_mixed.cu", "stage2d_fp32.cu", "batch_mixed.cu",
+                   "batch_fp32.cu"}
 FAST_FP32_FLAGS = ["-prec-div=false", "-prec-sqrt=false"]
 
 

@@ -41,6 +41,12 @@ cudaError_t launch_stage_learned_fp32(int, unsigned, size_t, cudaStream_t, const
 cudaError_t launch_stage_rk3_fp64(int, unsigned, size_t, cudaStream_t, const Geo&, const StageArgs&, const TmaMaps&);
 cudaError_t launch_stage_rk3_mixed(int, unsigned, size_t, cudaStream_t, const Geo&, const StageArgs&, const TmaMaps&);
 cudaError_t launch_stage_rk3_fp32(int, unsigned, size_t, cudaStream_t, const Geo&, const StageArgs&, const TmaMaps&);
+cudaError_t launch_stage_2d_fp64(int, int, int, unsigned, cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t launch_stage_2d_mixed(int, int, int, unsigned, cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t launch_stage_2d_fp32(int, int, int, unsigned, cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t set_smem_2d_fp64(int, int, bool);
+cudaError_t set_smem_2d_mixed(int, int, bool);
+cudaError_t set_smem_2d_fp32(int, int, bool);
 cudaError_t set_smem_rk3_fp64(size_t);
 cudaError_t set_smem_rk3_mixed(size_t);
 cudaError_t set_smem_rk3_fp32(size_t);
@@ -61,6 +67,14 @@ cudaError_t launch_stage(int prec, int stage, int tx, int ty, unsigned nb, size_
                          const Geo& g, const StageArgs& a, const TmaMaps* tm) {
   static const TmaMaps no_tma = {};
   const TmaMaps& maps = tm ? *tm : no_tma;
+  if (g.n[2] == 1 && g.bc[2] == 0 && g.recon == 0 && g.riemann != 2) {
+    // a two-dimensional box of a plain form: kernels of its own
+    switch (prec) {
+      case P_FP64: return launch_stage_2d_fp64(stage, tx, ty, nb, st, g, a);
+      case P_MIXED: return launch_stage_2d_mixed(stage, tx, ty, nb, st, g, a);
+      default: return launch_stage_2d_fp32(stage, tx, ty, nb, st, g, a);
+    }
+  }
   if (stage >= ST_RK3_1) {
     switch (prec) {
       case P_FP64: return launch_stage_rk3_fp64(stage, nb, smem, st, g, a, maps);
@@ -104,7 +118,17 @@ cudaError_t stage_set_smem_char(int prec, size_t bytes) {
     default: return set_smem_char_fp32(bytes);
   }
 }
+// the shared memory of the two-dimensional kernels, which size it themselves
+static cudaError_t stage_set_smem_2d(int prec, int tx, int ty, bool rk3) {
+  switch (prec) {
+    case P_FP64: return set_smem_2d_fp64(tx, ty, rk3);
+    case P_MIXED: return set_smem_2d_mixed(tx, ty, rk3);
+    default: return set_smem_2d_fp32(tx, ty, rk3);
+  }
+}
 cudaError_t stage_set_smem_rk3(int prec, size_t bytes) {
+  const cudaError_t e = stage_set_smem_2d(prec, 16, 8, true);
+  if (e != cudaSuccess) return e;
   switch (prec) {
     case P_FP64: return set_smem_rk3_fp64(bytes);
     case P_MIXED: return set_smem_rk3_mixed(bytes);
@@ -119,6 +143,8 @@ cudaError_t stage_set_smem_learned(int prec, size_t bytes) {
   }
 }
 cudaError_t stage_set_smem(int prec, int tx, int ty, size_t bytes) {
+  const cudaError_t e = stage_set_smem_2d(prec, tx, ty, false);
+  if (e != cudaSuccess) return e;
   switch (prec) {
     case P_FP64: return set_smem_fp64(tx, ty, bytes);
     case P_MIXED: return set_smem_mixed(tx, ty, bytes);

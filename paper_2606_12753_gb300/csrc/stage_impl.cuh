@@ -33,9 +33,14 @@ namespace mhd {
 // halo; 4 makes a ring row start 4 cells left of the tile, so that a plane
 // of 4-byte primitives can arrive as one TMA box whose first column (x =
 // tile origin - 4, a multiple of 4) meets the 16-byte rule of tensor copies.
-template <int TX, int TY, int XO = 2>
+// FLAT: the layout of a two-dimensional box's kernel, which holds one plane
+// of everything and no z-fluxes of the hydro variables (29 KB instead of 75
+// for a 16 x 8 tile of 4-byte primitives).
+template <int TX, int TY, int XO = 2, bool FLAT = false>
 struct Tile {
   static constexpr int XOFF = XO;
+  static constexpr int nPlanes = FLAT ? 1 : 4;   // ring slots
+  static constexpr int nPar = FLAT ? 1 : 2;      // copies of what is kept by plane parity
   static constexpr int W = TX + 2 * XO, H = TY + 4;
   static constexpr int nR = W * H;
   // lower-face normal fields of a plane: rows -1..TY of the ring (the rows
@@ -49,18 +54,19 @@ struct Tile {
   static constexpr int nC = TX * TY;
   // offsets in units of R
   static constexpr int oP = 0;
-  static constexpr int oBN = oP + 4 * 8 * nR;
-  static constexpr int oHX = oBN + 2 * nBslot;
+  static constexpr int oBN = oP + nPlanes * 8 * nR;
+  static constexpr int oHX = oBN + nPar * nBslot;
   static constexpr int oHY = oHX + 5 * nX;
   static constexpr int oHZ = oHY + 5 * nY;
-  static constexpr int oXC = oHZ + 5 * nZ;
-  static constexpr int oYC = oXC + 2 * 3 * nX;
-  static constexpr int oZC = oYC + 2 * 3 * nY;
+  static constexpr int oXC = oHZ + (FLAT ? 0 : 5 * nZ);
+  static constexpr int oYC = oXC + nPar * 3 * nX;
+  static constexpr int oZC = oYC + nPar * 3 * nY;
   static constexpr int oEC = oZC + 3 * nZ;
-  static constexpr int oEXY = oEC + 2 * 3 * nZ;
-  static constexpr int oEZ = oEXY + 2 * 2 * nE;
+  static constexpr int oEXY = oEC + nPar * 3 * nZ;
+  static constexpr int oEZ = oEXY + nPar * 2 * nE;
   static constexpr int oDU = oEZ + nE;
-  static constexpr int nRtot = oDU + 2 * 5 * nC;
+  static constexpr int nRtot = oDU + nPar * 5 * nC;
+  static constexpr int nHydro = 5 * (nX + nY + (FLAT ? 0 : nZ));   // R values of the hydro flux arrays
   // flux items of one plane: z-faces, x-faces, y-faces; the learned switch
   // queues their indices (unsigned short) in a region of its own
   static constexpr int nItems = nZ + nX + nY;
@@ -71,7 +77,7 @@ struct Tile {
   // per-cell half slopes (type R) over the (TX+2) x (TY+2) cells the faces touch:
   // x and y slopes of the current plane, z slopes of two planes (by parity)
   static constexpr int nSl = 7 * nZ;
-  static constexpr int nSlope = 4 * nSl;
+  static constexpr int nSlope = (FLAT ? 2 : 4) * nSl;   // (a flat tile has no z slopes)
   // byte offsets of the regions after the R arrays: the learned switch's
   // queue (QUEUE only), the int tables, the mbarriers
   template <typename R, bool QUEUE>
@@ -166,30 +172,40 @@ constexpr bool slopes_in_smem() {
   return MODE == FM_CHAR || (PREC == P_FP64 && MODE == FM_PLAIN && TX * TY <= 128);
 }
 
+// Which boxes a kernel advances: any (the batch, learned-switch and
+// characteristic kernels), or one single box of the plain forms, three- or
+// two-dimensional (one periodic z cell).  The last two are kernels of their
+// own, each without the other's code.  A two-dimensional box in the kernel of
+// any box paid for the ring, the second copies of everything kept by plane
+// parity and one FP64 CTA per SM instead of two (HLL 3200^2 mixed, stage 1 / 2:
+// 1855 / 2066 us there, 1643 / 2014 here; Orszag-Tang 512^2 FP64: 794 / 841
+// and 632 / 679).
+enum BoxKind { BOX_ANY = 0, BOX_3D = 1, BOX_2D = 2 };
+
 // Whether a kernel takes interior planes by TMA: the plain single-box stage
 // kernels with 4-byte primitives (mixed, FP32).  The batch kernel gathers
 // every plane: its small outflow boxes have few interior tiles, and a tensor
 // map needs rows that are a multiple of 16 bytes, which few of its boxes of
 // arbitrary width have.
-template <int PREC, int MODE, bool SINGLE_BOX>
+template <int PREC, int MODE, int KIND>
 __host__ __device__ constexpr bool tma_planes() {
-  return SINGLE_BOX && PREC != P_FP64 && MODE == FM_PLAIN;
+  return KIND == BOX_3D && PREC != P_FP64 && MODE == FM_PLAIN;
 }
 
 // Whether a kernel solves, on a tile that the box edge cuts, only the flux
 // items its valid cells need (a per-tile list in shared memory, in the
 // learned switch's queue region): the batch kernel's plain forms without a
 // slope phase, whose boxes of arbitrary size leave many ragged tiles.
-template <int PREC, int MODE, bool SINGLE_BOX, int TX, int TY>
+template <int PREC, int MODE, int KIND, int TX, int TY>
 __host__ __device__ constexpr bool compact_items() {
-  return !SINGLE_BOX && MODE == FM_PLAIN && !slopes_in_smem<PREC, MODE, TX, TY>();
+  return KIND == BOX_ANY && MODE == FM_PLAIN && !slopes_in_smem<PREC, MODE, TX, TY>();
 }
 
 // Ring x-offset of a kernel: kernels with TMA planes pad the ring rows (see
 // Tile); all others keep the 2-cell halo.
-template <int PREC, int MODE, bool SINGLE_BOX>
+template <int PREC, int MODE, int KIND>
 __host__ __device__ constexpr int ring_xo() {
-  return tma_planes<PREC, MODE, SINGLE_BOX>() ? 4 : 2;
+  return tma_planes<PREC, MODE, KIND>() ? 4 : 2;
 }
 
 // SPLIT: the update phase splits each cell between two threads (face group
@@ -201,7 +217,7 @@ __host__ __device__ constexpr int ring_xo() {
 // split there.  PREFETCH (split form only): phase D's stored values are
 // loaded into registers before phase C.
 template <int PREC, int STAGE, int TX, int TY, int MODE = FM_PLAIN, bool SPLIT = false, bool PREFETCH = false,
-          bool SINGLE_BOX = false>
+          int KIND = BOX_ANY>
 struct StageKernel {
   static constexpr bool LEARN = MODE == FM_LEARNED;
   static constexpr bool CHAR = MODE == FM_CHAR;
@@ -209,13 +225,14 @@ struct StageKernel {
   using R = typename Prec<PREC>::R;
   using S = typename Prec<PREC>::S;
   using K = typename Prec<PREC>::K;
-  using T = Tile<TX, TY, ring_xo<PREC, MODE, SINGLE_BOX>()>;
+  static constexpr bool FLAT = KIND == BOX_2D;
+  using T = Tile<TX, TY, ring_xo<PREC, MODE, KIND>(), FLAT>;
   static constexpr int W = T::W;
   static constexpr int XO = T::XOFF;
   // TMA planes: plain kernels with 4-byte primitives
-  static constexpr bool kTMA = tma_planes<PREC, MODE, SINGLE_BOX>();
+  static constexpr bool kTMA = tma_planes<PREC, MODE, KIND>();
   static constexpr bool kDyn = !SPLIT && MODE != FM_LEARNED;   // dynamic flux or slope phase (see fluxes)
-  static constexpr bool kCompact = kDyn && compact_items<PREC, MODE, SINGLE_BOX, TX, TY>();   // see build_items
+  static constexpr bool kCompact = kDyn && compact_items<PREC, MODE, KIND, TX, TY>();   // see build_items
   static constexpr bool kQueue = LEARN || kCompact;   // the layout's queue region is in use
   static constexpr int kLoadBarrier = 2, kPlaneBarrier = 3;            // named barriers of that form
   static_assert(!kTMA || ((8 * T::nR * sizeof(R)) % 128 == 0 && (T::oBN * sizeof(R)) % 128 == 0 &&
@@ -407,6 +424,11 @@ struct StageKernel {
     }
   }
 
+  static __device__ __forceinline__ void solve(const Geo& g, const R* wl, const R* wr, R bn, R gam, R ig, R* f, R* cm) {
+    if (g.riemann == 1) hll_flux_g(wl, wr, bn, gam, ig, f, cm);
+    else hlld_flux_g(wl, wr, bn, gam, ig, f, cm);
+  }
+
   // one flux item of phase B: reconstruction, Riemann flux, store
   static __device__ __forceinline__ void flux_item(const Geo& g, R* sm, int k, int q, int nZ, int w, R gam, R ig) {
     {
@@ -416,15 +438,13 @@ struct StageKernel {
         R bnc[2];
         const int D = item_stencil(sm, k, q, nZ, w, c, bn, o, bnc);
         plm_face_char(c[0], c[1], c[2], c[3], bnc[0], bnc[1], gam, wl, wr, gpar<R>(g.rho_floor, g.frho_floor), gpar<R>(g.p_floor, g.fp_floor));
-        if (g.riemann == 1) hll_flux_g(wl, wr, bn, gam, ig, f, &cm);
-        else hlld_flux_g(wl, wr, bn, gam, ig, f, &cm);
+        solve(g, wl, wr, bn, gam, ig, f, &cm);
         store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
         return;
       }
       const int D = item_stencil(sm, k, q, nZ, w, c, bn, o);
       plm_face(c[0], c[1], c[2], c[3], wl, wr, gpar<R>(g.rho_floor, g.frho_floor), gpar<R>(g.p_floor, g.fp_floor));
-      if (g.riemann == 1) hll_flux_g(wl, wr, bn, gam, ig, f, &cm);
-      else hlld_flux_g(wl, wr, bn, gam, ig, f, &cm);
+      solve(g, wl, wr, bn, gam, ig, f, &cm);
       store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
     }
   }
@@ -547,11 +567,44 @@ struct StageKernel {
       wr[0] = rmax(wr[0], gpar<R>(g.rho_floor, g.frho_floor));
       wl[4] = rmax(wl[4], gpar<R>(g.p_floor, g.fp_floor));
       wr[4] = rmax(wr[4], gpar<R>(g.p_floor, g.fp_floor));
-      if (g.riemann == 1) hll_flux_g(wl, wr, bn, gam, ig, f, &cm);
-      else hlld_flux_g(wl, wr, bn, gam, ig, f, &cm);
+      solve(g, wl, wr, bn, gam, ig, f, &cm);
       store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
     }
     cell_emf(sm, q, threadIdx.x, blockDim.x);
+  }
+
+  // The z-faces of a two-dimensional box: both states are the cell's own
+  // (its z slopes vanish) and only their EMFs and mass flux are read.  The
+  // solution is kept whole and its two states apart in the compiler's eyes:
+  // where the out-of-plane field vanishes, the EMFs are rounding alone, and a
+  // solution with its dead parts removed rounds differently (its products
+  // fuse differently) without being faster.  The items run from the last
+  // thread down: the first threads have the longer share of the x- and
+  // y-faces.
+  static __device__ __forceinline__ float opaque(float x) { asm volatile("" : "+f"(x)); return x; }
+  static __device__ __forceinline__ double opaque(double x) { asm volatile("" : "+d"(x)); return x; }
+  static __device__ __forceinline__ void zfaces_2d(const Geo& g, R* sm) {
+    const R gam = gpar<R>(g.gamma, g.fgamma);
+    const R ig = R(1) / (gam - R(1));
+    R* C = sm + T::oZC;
+    for (int w = (int)blockDim.x - 1 - (int)threadIdx.x; w < T::nZ; w += blockDim.x) {
+      const int i = w % (TX + 2) - 1, j = w / (TX + 2) - 1;
+      const int r = MHD_SIDX((i + XO) + W * (j + 2), T::nR);
+      R c[7], f[7], cm;
+      gather<2>(sm + T::oP, T::nR, r, c);
+      const R bn = bn_slot(sm, 0)[2 * T::nB + MHD_SIDX(bn_of(r), T::nB)];
+      c[0] = rmax(c[0], gpar<R>(g.rho_floor, g.frho_floor));
+      c[4] = rmax(c[4], gpar<R>(g.p_floor, g.fp_floor));
+      R d[7];
+#pragma unroll
+      for (int v = 0; v < 7; ++v) d[v] = opaque(c[v]);
+      solve(g, c, d, bn, gam, ig, f, &cm);
+#pragma unroll
+      for (int v = 1; v < 5; ++v) f[v] = opaque(f[v]);
+      C[w] = -f[5];
+      C[T::nZ + w] = f[6];
+      C[2 * T::nZ + w] = oriented_mass_flux(f[0], c[0], c[0], cm, gpar<R>(g.deadband, g.fdeadband));
+    }
   }
 
   // cell-centred E_c = -v x B_c of plane q
@@ -804,8 +857,8 @@ struct StageKernel {
     }
   }
 
-  // Phase C of a two-dimensional box (one periodic z cell).  The flux pass
-  // computed the x/y data of plane 1, which is plane 0 itself, into slot 1;
+  // Phase C of a two-dimensional box (one periodic z cell).  Kernels of any
+  // box run the flux pass as plane 1, which is plane 0 itself, into slot 1;
   // the z-faces below and above a cell are one face, so the divergence drops
   // their difference (exactly zero), and the edges E_x, E_y at k-1/2 and
   // k+1/2 are one set, written to both slots.
@@ -829,14 +882,15 @@ struct StageKernel {
                              (HY[v * T::nY + iyp] - HY[v * T::nY + iym]) * idy;
     }
     const bool mean = g.emf_mean != 0;
-    const R* XC = sm + T::oXC + 3 * T::nX;
-    const R* YC = sm + T::oYC + 3 * T::nY;
+    constexpr int slot = FLAT ? 0 : 1;
+    const R* XC = sm + T::oXC + slot * 3 * T::nX;
+    const R* YC = sm + T::oYC + slot * 3 * T::nY;
     const R* ZC = sm + T::oZC;
-    const R* EC = sm + T::oEC + 3 * T::nZ;
+    const R* EC = sm + T::oEC + slot * 3 * T::nZ;
     R* EZ = sm + T::oEZ;
     R* EX0 = sm + T::oEXY;
     R* EY0 = EX0 + T::nE;
-    R* EX1 = sm + T::oEXY + 2 * T::nE;
+    R* EX1 = sm + T::oEXY + slot * 2 * T::nE;
     R* EY1 = EX1 + T::nE;
     constexpr int nX = T::nX, nY = T::nY, nZ = T::nZ;
     for (int e = threadIdx.x; e < T::nE; e += apart ? kEdgeThreads : (int)blockDim.x) {
@@ -990,7 +1044,7 @@ struct StageKernel {
     const R* EZ = sm + T::oEZ;
     const R* EX0 = sm + T::oEXY + (k & 1) * 2 * T::nE;         // k-1/2
     const R* EY0 = EX0 + T::nE;
-    const R* EX1 = sm + T::oEXY + ((k + 1) & 1) * 2 * T::nE;   // k+1/2
+    const R* EX1 = sm + T::oEXY + (FLAT ? 0 : (k + 1) & 1) * 2 * T::nE;   // k+1/2
     const R* EY1 = EX1 + T::nE;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const bool outx = g.bc[0] == 1, outy = g.bc[1] == 1, outz = g.bc[2] == 1;
@@ -1117,25 +1171,23 @@ struct StageKernel {
 
   // zc: the face group's z-face carry (split form; reset at a chunk's
   // first plane); pre: the values prefetch() fetched for this plane (nullptr:
-  // none were).  single_plane: the item's only plane (a two-dimensional box),
-  // which no flux phase follows: the single-box mixed and FP64 kernels split
-  // its cells between two threads even in the one-pass form, whose other
-  // threads would otherwise idle there.
+  // none were).  The mixed and FP64 kernels of a single two-dimensional box,
+  // whose only plane no flux phase follows, split its cells between two
+  // threads too: the others would idle there.
   static constexpr bool kCanSplit =
-      SPLIT || (SINGLE_BOX && PREC != P_FP32 && T::nC % 32 == 0 &&
-                (size_t)5 * T::nC * sizeof(double) <= (size_t)5 * (T::nX + T::nY + T::nZ) * sizeof(R));
+      SPLIT || (FLAT && PREC != P_FP32 && T::nC % 32 == 0 &&
+                (size_t)5 * T::nC * sizeof(double) <= (size_t)T::nHydro * sizeof(R));
   static __device__ __forceinline__ void update_plane(const Geo& g, const StageArgs& a, R* sm, const StepDt& dt,
                                                       int gi0, int gj0, int k, unsigned& nrho, unsigned& np,
-                                                      bool& bad, R& smax, ZCarry& zc, const Pre* pre = nullptr,
-                                                      bool single_plane = false) {
+                                                      bool& bad, R& smax, ZCarry& zc, const Pre* pre = nullptr) {
     const R* DU = sm + T::oDU + (k & 1) * 5 * T::nC;
     const int nx = g.n[0], ny = g.n[1];
     const int t = threadIdx.x;
     if constexpr (kCanSplit) {
-      if (SPLIT || (single_plane && 2 * T::nC <= (int)blockDim.x)) {
+      if (SPLIT || 2 * T::nC <= (int)blockDim.x) {
       static_assert(T::nC % 32 == 0, "the split update phase needs whole warps per group");
       double* U5 = reinterpret_cast<double*>(sm + T::oHX);   // [5][nC], in the idle flux arrays
-      static_assert((size_t)5 * T::nC * sizeof(double) <= (size_t)5 * (T::nX + T::nY + T::nZ) * sizeof(R),
+      static_assert((size_t)5 * T::nC * sizeof(double) <= (size_t)T::nHydro * sizeof(R),
                     "hand-over does not fit in the flux arrays");
       if (t >= 2 * T::nC) return;
       const int c = t < T::nC ? t : t - T::nC;
@@ -1296,7 +1348,27 @@ struct StageKernel {
     bool bad = false;
     R smax = R(0);
 
-    if (g.n[2] == 1 && g.bc[2] == 0) {
+    if constexpr (FLAT) {
+      // one plane: x- and y-slopes and fluxes, and the z-faces' EMFs
+      load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, 0, true);
+      __syncthreads();
+      if constexpr (SLOPES) {
+        for (int it = threadIdx.x; it < 2 * T::nZ; it += blockDim.x) slope_item(g, sm, sl, 0, it);
+        __syncthreads();
+        fluxes_sl(g, sm, sl, 0, 0, false);
+      } else {
+        fluxes(g, sm, 0, 0, false, nullptr);   // all threads start together: static items
+      }
+      zfaces_2d(g, sm);
+      __syncthreads();
+      edges_2d(g, sm);
+      __syncthreads();
+      ZCarry zc{S(0), R(0), false};
+      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc);
+      finish(a, nrho, np, nh, nd, bad, smax);
+      fold_bounds_flag(a);
+    } else {
+    if (KIND == BOX_ANY && g.n[2] == 1 && g.bc[2] == 0) {
       // A two-dimensional box (one periodic z cell): every ring slot holds
       // plane 0, so one flux pass (the z-faces, which feed E_x and E_y, and
       // the x/y faces of the plane) replaces the chunk prologue and the
@@ -1329,7 +1401,7 @@ struct StageKernel {
       edges_2d(g, sm);
       __syncthreads();
       ZCarry zc{S(0), R(0), false};
-      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc, nullptr, true);
+      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc);
       finish(a, nrho, np, nh, nd, bad, smax);
       fold_bounds_flag(a);
       return;
@@ -1423,6 +1495,7 @@ struct StageKernel {
     finish(a, nrho, np, nh, nd, bad, smax);
     if (ntma && threadIdx.x == 0) atomicAdd(&a.counters[C_TMA], (unsigned long long)ntma);
     fold_bounds_flag(a);
+    }
   }
 
   // bounds-checked build: the CTA's shared-memory index flag into the status word
@@ -1449,12 +1522,27 @@ __host__ __device__ constexpr int stage_min_blocks() {
   return PREC == P_FP64 ? (TX * TY <= 64 ? 2 : 1) : 768 / stage_threads<PREC, TX, TY>();
 }
 
+// CTAs per SM of the kernel of a two-dimensional box: its flat tile leaves the
+// shared memory of a second FP64 CTA.
+template <int PREC, int TX, int TY>
+__host__ __device__ constexpr int stage2d_min_blocks() {
+  return PREC == P_FP64 ? (TX * TY <= 128 ? 2 : 1) : stage_min_blocks<PREC, TX, TY>();
+}
+
 template <int PREC, int STAGE, int TX, int TY>
 __global__ void __launch_bounds__(stage_threads<PREC, TX, TY>(), stage_min_blocks<PREC, TX, TY>())
     stage_kernel(Geo g, StageArgs a, const __grid_constant__ TmaMaps tm) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  StageKernel<PREC, STAGE, TX, TY, FM_PLAIN, false, false, true>::run_item(
+  StageKernel<PREC, STAGE, TX, TY, FM_PLAIN, false, false, BOX_3D>::run_item(
       g, a, blockIdx.x, smem_raw, &tm);
+}
+
+// The same stage of a two-dimensional box (one periodic z cell).
+template <int PREC, int STAGE, int TX, int TY>
+__global__ void __launch_bounds__(stage_threads<PREC, TX, TY>(), stage2d_min_blocks<PREC, TX, TY>())
+    stage_kernel_2d(Geo g, StageArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  StageKernel<PREC, STAGE, TX, TY, FM_PLAIN, false, false, BOX_2D>::run_item(g, a, blockIdx.x, smem_raw);
 }
 
 // The same stage with the learned HLL/HLLD face switch.

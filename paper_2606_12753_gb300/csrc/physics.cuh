@@ -108,9 +108,24 @@ __host__ __device__ __forceinline__ double rsqrt_(double x) {   // square root
   return sqrt(x);
 #endif
 }
+// The same root one operation shorter: the refinement applied to x y0
+// (used where the result may round differently).
+__host__ __device__ __forceinline__ double root_(double x) {
+#ifdef __CUDA_ARCH__
+  if (!f64_plain(x) || __double2hiint(x) < 0) return sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double t = x * y;
+  const double h = fma(-t, y, 1.0);
+  return fma(t, h * fma(0.375, h, 0.5), t);
+#else
+  return sqrt(x);
+#endif
+}
 __host__ __device__ __forceinline__ float rcp_(float x) { return 1.0f / x; }
 __host__ __device__ __forceinline__ float rrsqrt_(float x) { return rsqrtf(x); }
 __host__ __device__ __forceinline__ float rsqrt_(float x) { return sqrtf(x); }
+__host__ __device__ __forceinline__ float root_(float x) { return sqrtf(x); }
 
 // Sign-bit helpers (integer operations: they keep the sign tests of the
 // limiter off the FP64 pipe).
@@ -139,6 +154,20 @@ __host__ __device__ __forceinline__ double fmin_(double a, double b) {
 }
 __host__ __device__ __forceinline__ float fmin_(float a, float b) { return fminf(a, b); }
 
+// A quarter of a non-negative value.  FP64 on the device: two off the
+// exponent, on the integer pipe (a multiplication would take a slot of the
+// FP64 pipe); zero, the smallest exponents, infinity and NaN multiply.
+__host__ __device__ __forceinline__ float quarter_(float x) { return 0.25f * x; }
+__host__ __device__ __forceinline__ double quarter_(double x) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi - 0x00300000u < 0x7ff00000u - 0x00300000u) return __hiloint2double((int)(hi - 0x00200000u), __double2loint(x));
+  return (hi | (unsigned)__double2loint(x)) == 0u ? x : 0.25 * x;
+#else
+  return 0.25 * x;
+#endif
+}
+
 // Half of the MC-limited slope of the middle of three values (a face takes
 // the cell value plus or minus it): with dm = q0 - qm and dp = qp - q0, the MC
 // slope is sign(dp) min(2|dm|, 2|dp|, |dm+dp|/2) when dm and dp have the same
@@ -149,7 +178,7 @@ __host__ __device__ __forceinline__ float fmin_(float a, float b) { return fminf
 // underflow).
 template <typename R>
 __host__ __device__ __forceinline__ R mc_lim_half(R dm, R dp) {
-  R m = fmin_(fmin_(rabs(dm), rabs(dp)), R(0.25) * rabs(dm + dp));
+  R m = fmin_(fmin_(rabs(dm), rabs(dp)), quarter_(rabs(dm + dp)));
   m = opposite_signs(dm, dp) ? R(0) : m;
   return copysign_(m, dp);
 }
@@ -355,12 +384,228 @@ __host__ __device__ __forceinline__ void hlld_flux(const R* wl, const R* wr, R b
   hlld_flux_g(wl, wr, bn, gamma, R(1) / (gamma - R(1)), f, cmax);
 }
 
+// ---------------------------------------------------------------------------
+// The same two solvers with fewer operations: the forms of the FP64 kernels,
+// which are bound by the FP64 pipe (one warp-instruction per ~17 SM cycles,
+// the other pipes nearly idle).  They equal the forms above up to rounding
+// and are the nearer ones to the exact flux (random faces against 80-bit
+// arithmetic: HLLD 2.6e-17 of the flux scale on the mean against 6.1e-17,
+// HLL 2.2e-17 against 2.4e-17).  FP32 fluxes keep the forms above: a change
+// of FP32 rounding flips limiter and upwind choices here and there, which
+// moves single cells by 1e-3.  Per face an HLLD solution takes about 160 FP64
+// operations instead of 250, by these identities:
+//   * c_f^2 = T / (2 rho), T = gamma p + |B|^2 + sqrt((gamma p - |B|^2)^2 + 4 gamma p |B_t|^2):
+//     the larger of two fast speeds is found by comparing T_L rho_R with
+//     T_R rho_L, and one division and one outer root serve both states;
+//   * the flux of every region has the form of the physical flux of that
+//     region's state with its total pressure, so one evaluation on the
+//     selected state replaces F + S (U* - U) + S* (U** - U*);
+//   * rho* and sqrt(rho*) follow from one reciprocal root y of
+//     m (S - S_M), m = rho (S - u): sqrt(rho*) = |m| y, 1/sqrt(rho*) = |S - S_M| y;
+//   * across an Alfven wave v** - v* = +-sgn(bn) (B** - B*)/sqrt(rho*);
+//   * only the side of S_M that holds the face forms its energy, and the
+//     other side's star state is formed only where a double-star state needs it.
+// Measured (GB300, 128^3, stage 1 / 2 in us): HLLD 7197 / 7678 with the plain
+// solvers, 5521 / 5984 with these; HLL 5487 / 5967 and 5031 / 5515.
+
+// x with its sign flipped where f is set (on the integer pipe in FP64)
+__host__ __device__ __forceinline__ double flip_(double x, bool f) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(x) ^ (f ? (int)0x80000000 : 0), __double2loint(x));
+#else
+  return f ? -x : x;
+#endif
+}
+
+// The larger fast speed of two states, b2_* = |B|^2 and bt2_* = |B_t|^2 of each.
+__host__ __device__ __forceinline__ double max_fast_speed(const double* wl, const double* wr, double b2_l, double b2_r,
+                                                          double bt2_l, double bt2_r, double gamma) {
+  const double g4 = 4.0 * gamma;
+  const double x_l = gamma * wl[4] - b2_l, x_r = gamma * wr[4] - b2_r;
+  const double t_l = gamma * wl[4] + b2_l + root_(x_l * x_l + (g4 * wl[4]) * bt2_l);
+  const double t_r = gamma * wr[4] + b2_r + root_(x_r * x_r + (g4 * wr[4]) * bt2_r);
+  const bool l = lt_(t_r * wl[0], t_l * wr[0]);
+  const double t = l ? t_l : t_r, rho = l ? wl[0] : wr[0];
+  // sqrt(t / (2 rho)) = t / sqrt(2 rho t)
+  return t * (0.70710678118654752440 * rrsqrt_(rho * t));
+}
+
+// Whether a star state's denominator den = num - bn^2 counts as zero:
+// |den| <= eps max(|num|, bn^2), as in star_side.  On the device, where
+// the exponents already put |den| above 2^-38 bn^2, and so (|num| <= |den| +
+// bn^2) above 1e-12 of both, no FP64 operation is needed.
+__host__ __device__ __forceinline__ bool star_degenerate(double den, double num, double bn2) {
+#ifdef __CUDA_ARCH__
+  const unsigned hd = (unsigned)__double2hiint(den) & 0x7fffffffu, hb = (unsigned)__double2hiint(bn2);
+  if (hd + (37u << 20) > hb) return false;
+#endif
+  return le_(rabs(den), Eps<double>::degen * rmax(rabs(num), bn2));
+}
+
+// Star state of one side as the lean solver needs it: m = rho (S - u), ssm =
+// S - S_M, smu = S_M - u.
+struct LeanStar {
+  double v, w, by, bz, sq, isq, y;   // sq = sqrt(rho*), isq = 1/sqrt(rho*), y = 1/sqrt(m ssm)
+  bool degen;
+};
+__host__ __device__ __forceinline__ LeanStar lean_star(double v, double w, double by, double bz, double bn, double bn2,
+                                                       double m, double ssm, double smu) {
+  LeanStar st;
+  const double num = m * ssm, den = num - bn2;
+  st.degen = star_degenerate(den, num, bn2);
+  const double t = smu * rcp_(den);
+  const double c1 = st.degen ? 0.0 : bn * t;          // v* = v - B_t c1
+  const double c2 = st.degen ? 1.0 : 1.0 + m * t;    // B_t* = B_t c2, c2 = (m (S - u) - bn^2) / den
+  st.v = v - by * c1;
+  st.w = w - bz * c1;
+  st.by = by * c2;
+  st.bz = bz * c2;
+  st.y = rrsqrt_(num);
+  st.sq = rabs(m) * st.y;
+  st.isq = rabs(ssm) * st.y;
+  return st;
+}
+
+// Flux of the state (rho, u, v, w, energy e, total pressure pt, transverse
+// field by, bz, vb = v.B).
+__host__ __device__ __forceinline__ void state_flux(double rho, double u, double v, double w, double e, double pt,
+                                                    double by, double bz, double vb, double bn, double bn2, double* f) {
+  const double mu = rho * u;
+  f[0] = mu;
+  f[1] = mu * u + (pt - bn2);
+  f[2] = mu * v - bn * by;
+  f[3] = mu * w - bn * bz;
+  f[4] = (e + pt) * u - bn * vb;
+  f[5] = u * by - bn * v;
+  f[6] = u * bz - bn * w;
+}
+
+// Conserved hydro values and flux of one outer state.
+__host__ __device__ __forceinline__ void lean_side(const double* w, double bn, double bn2, double b2, double ig,
+                                                   double* u, double* f) {
+  const double e = w[4] * ig + 0.5 * (w[0] * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) + b2);
+  const double vb = w[1] * bn + w[2] * w[5] + w[3] * w[6];
+  state_flux(w[0], w[1], w[2], w[3], e, w[4] + 0.5 * b2, w[5], w[6], vb, bn, bn2, f);
+  u[0] = w[0];
+  u[1] = f[0];
+  u[2] = w[0] * w[2];
+  u[3] = w[0] * w[3];
+  u[4] = e;
+}
+
+// HLLD flux; ig = 1/(gamma - 1).  Regions, ties and the degenerate star state
+// as hlld_flux_g: a degenerate side keeps its outer tangential values, and
+// its transverse induction flux the outer velocity.
+__host__ __device__ __forceinline__ void hlld_flux_lean(const double* wl, const double* wr, double bn, double gamma,
+                                                        double ig, double* f, double* cmax) {
+  const double bn2 = bn * bn;
+  const double bt2l = wl[5] * wl[5] + wl[6] * wl[6], bt2r = wr[5] * wr[5] + wr[6] * wr[6];
+  const double b2l = bn2 + bt2l, b2r = bn2 + bt2r;
+  const double ptl = wl[4] + 0.5 * b2l, ptr = wr[4] + 0.5 * b2r;
+  const double cm = max_fast_speed(wl, wr, b2l, b2r, bt2l, bt2r, gamma);
+  *cmax = cm;
+  const double sl = rmin(wl[1], wr[1]) - cm, sr = rmax(wl[1], wr[1]) + cm;
+  const bool out_l = gt0(sl), outside = out_l || lt0(sr);
+  // the outer sides' S - u, m = rho (S - u) and the contact speed S_M
+  const double sdl = sl - wl[1], sdr = sr - wr[1];
+  const double ml = wl[0] * sdl, mr = wr[0] * sdr;
+  const double sm = ((ptl - ptr) + mr * wr[1] - ml * wl[1]) * rcp_(mr - ml);
+  const bool left = outside ? out_l : ge0(sm);
+  // A: the side that holds the face, B: the other one
+  const double rho = left ? wl[0] : wr[0], u = left ? wl[1] : wr[1], p = left ? wl[4] : wr[4];
+  const double va = left ? wl[2] : wr[2], wa = left ? wl[3] : wr[3];
+  const double bya = left ? wl[5] : wr[5], bza = left ? wl[6] : wr[6];
+  const double b2 = left ? b2l : b2r, pta = left ? ptl : ptr;
+  const double vb = u * bn + va * bya + wa * bza;
+  const double e = p * ig + 0.5 * (rho * (u * u + va * va + wa * wa) + b2);
+  // the state whose flux this is
+  double fr = rho, fu = u, fv = va, fw = wa, fby = bya, fbz = bza, fe = e, fvb = vb, fpt = pta;
+  double smu = 0.0;
+  bool degen = false;
+  if (!outside) {
+    const double s = left ? sl : sr, m = left ? ml : mr, sd = left ? sdl : sdr;
+    const double ssm = s - sm;
+    smu = sm - u;
+    const LeanStar A = lean_star(va, wa, bya, bza, bn, bn2, m, ssm, smu);
+    degen = A.degen;
+    const double inv = A.y * A.y * m;   // 1 / (S - S_M)
+    fpt = pta + m * smu;
+    fr = m * inv;
+    fu = sm;
+    const double smbn = sm * bn;
+    fvb = smbn + A.v * A.by + A.w * A.bz;
+    fe = (sd * e - pta * u + fpt * sm + bn * (vb - fvb)) * inv;
+    fv = A.v;
+    fw = A.w;
+    fby = A.by;
+    fbz = A.bz;
+    // beyond the Alfven wave of side A: S*_L < 0 (left), S*_R >= 0 (right)
+    const double al = rabs(bn) * A.isq;
+    if (left ? lt_(sm, al) : le_(-sm, al)) {
+      const double sb = left ? sr : sl;
+      const LeanStar B = lean_star(left ? wr[2] : wl[2], left ? wr[3] : wl[3], left ? wr[5] : wl[5],
+                                      left ? wr[6] : wl[6], bn, bn2, left ? mr : ml, sb - sm,
+                                      sm - (left ? wr[1] : wl[1]));
+      const bool neg = lt0(bn) == left;   // sign of sgn(bn) (+ on the left, - on the right)
+      const double is = rcp_(A.sq + B.sq);
+      const double ps = flip_(A.sq * B.sq, neg);
+      fby = (A.sq * B.by + B.sq * A.by + ps * (B.v - A.v)) * is;
+      fbz = (A.sq * B.bz + B.sq * A.bz + ps * (B.w - A.w)) * is;
+      const double k = flip_(A.isq, neg);
+      fv = A.v + k * (fby - A.by);
+      fw = A.w + k * (fbz - A.bz);
+      const double vbs = fvb;
+      fvb = smbn + fv * fby + fw * fbz;
+      fe = fe - flip_(A.sq, neg) * (vbs - fvb);
+    }
+  }
+  state_flux(fr, fu, fv, fw, fe, fpt, fby, fbz, fvb, bn, bn2, f);
+  if (degen) {   // outside the star region degen is false
+    f[5] -= smu * bya;
+    f[6] -= smu * bza;
+  }
+}
+
+// HLL flux a F_L + b F_R + c (U_R - U_L) with the three weights formed once.
+__host__ __device__ __forceinline__ void hll_flux_lean(const double* wl, const double* wr, double bn, double gamma,
+                                                       double ig, double* f, double* cmax) {
+  const double bn2 = bn * bn;
+  const double bt2l = wl[5] * wl[5] + wl[6] * wl[6], bt2r = wr[5] * wr[5] + wr[6] * wr[6];
+  const double b2l = bn2 + bt2l, b2r = bn2 + bt2r;
+  const double cm = max_fast_speed(wl, wr, b2l, b2r, bt2l, bt2r, gamma);
+  *cmax = cm;
+  const double sl = rmin(wl[1], wr[1]) - cm, sr = rmax(wl[1], wr[1]) + cm;
+  const double is = rcp_(sr - sl);
+  double a = sr * is, b = -(sl * is), c = sl * a;
+  if (ge0(sl)) { a = 1.0; b = c = 0.0; }   // outside the fan: one side's flux
+  else if (le0(sr)) { b = 1.0; a = c = 0.0; }
+  double ul[5], ur[5], fl[7], fr[7];
+  lean_side(wl, bn, bn2, b2l, ig, ul, fl);
+  lean_side(wr, bn, bn2, b2r, ig, ur, fr);
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const double du = q < 5 ? ur[q] - ul[q] : wr[q] - wl[q];
+    f[q] = a * fl[q] + (b * fr[q] + c * du);
+  }
+}
+
 // Mass flux that orients the upwind EMF average: the face mass flux, or 0
 // when it lies inside a rounding deadband eps (rho_L + rho_R)/2 c_max, so
 // rounding noise of a vanishing mass flux selects the mean of both sides
 // instead of an arbitrary side.
+// FP64 on the device: where the exponents already put |f0| above the band
+// (eps (rho_L + rho_R)/2 c_max < 2^(sum of the exponents + 3)), no FP64
+// operation is needed.
 template <typename R>
 __host__ __device__ __forceinline__ R oriented_mass_flux(R f0, R rho_l, R rho_r, R cmax, R eps) {
+#ifdef __CUDA_ARCH__
+  if constexpr (sizeof(R) == 8) {
+    const int er = max(__double2hiint((double)rho_l), __double2hiint((double)rho_r));
+    const int ec = __double2hiint((double)cmax) >> 20, ee = __double2hiint((double)eps) >> 20;
+    const int band = (er >> 20) + ec + ee - 2 * 1023 + 3;
+    if (((__double2hiint((double)f0) & 0x7fffffff) >> 20) > band) return f0;
+  }
+#endif
   return le_(rabs(f0), eps * R(0.5) * (rho_l + rho_r) * cmax) ? R(0) : f0;
 }
 
@@ -400,7 +645,7 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
                                                     R* slope) {
   const R rho = w0[0];
   const R ir = rcp_(rho);
-  const R a2 = gamma * w0[4] * ir, a = rsqrt_(a2), sr = rsqrt_(rho), isr = rcp_(sr);
+  const R a2 = gamma * w0[4] * ir, a = root_(a2), sr = root_(rho), isr = rcp_(sr);
   const R bnr = bn0 * isr, b1 = w0[5] * isr, b2 = w0[6] * isr;
   const R bt2 = b1 * b1 + b2 * b2, bsq = bnr * bnr + bt2;
   // forms without cancellation: c_f^2 - c_s^2 = sqrt((a^2-b^2)^2 + 4 a^2 b_t^2),
@@ -413,9 +658,9 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
   const R sq = sqrt((a2 - bsq) * (a2 - bsq) + R(4) * a2 * bt2);
   const R cf2 = R(0.5) * (a2 + bsq + sq);
   const R cs2 = gt0(cf2) ? a2 * bnr * bnr * rcp_(cf2) : R(0);
-  const R cf = rsqrt_(cf2), cs = rsqrt_(cs2), bt = rsqrt_(bt2);
+  const R cf = root_(cf2), cs = root_(cs2), bt = root_(bt2);
   R be1, be2;
-  if (lt_(Eps<R>::degen * rsqrt_(a2 + bsq), bt)) {
+  if (lt_(Eps<R>::degen * root_(a2 + bsq), bt)) {
     const R ib = rcp_(bt);
     be1 = b1 * ib;
     be2 = b2 * ib;
@@ -426,8 +671,8 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
   if (lt_(Eps<R>::degen * cf2, sq)) {
     const R id = rcp_(sq);
     const R fa = R(0.5) * (bsq - a2 + sq), as2 = R(0.5) * (a2 - bsq + sq);   // c_f^2 - a^2, a^2 - c_s^2
-    af = rsqrt_((gt0(as2) ? as2 : R(0)) * id);
-    as = rsqrt_((gt0(fa) ? fa : R(0)) * id);
+    af = root_((gt0(as2) ? as2 : R(0)) * id);
+    as = root_((gt0(fa) ? fa : R(0)) * id);
   } else {
     af = R(1);
     as = R(0);

@@ -609,25 +609,48 @@ __host__ __device__ __forceinline__ R oriented_mass_flux(R f0, R rho_l, R rho_r,
   return le_(rabs(f0), eps * R(0.5) * (rho_l + rho_r) * cmax) ? R(0) : f0;
 }
 
-// Gardiner-Stone upwind selection by the sign of a face mass flux.
+// Gardiner-Stone upwind selection by the sign of a face mass flux: the
+// difference lo_a - lo_b of one side, hi_a - hi_b of the other, or their mean.
 template <typename R>
-__host__ __device__ __forceinline__ R upwind(R m, R lo, R hi) {
+__host__ __device__ __forceinline__ R upwind(R m, R lo_a, R lo_b, R hi_a, R hi_b) {
+  const R lo = lo_a - lo_b, hi = hi_a - hi_b;
   return gt0(m) ? lo : (lt0(m) ? hi : R(0.5) * (lo + hi));
+}
+// The same for a mass flux that is not zero: select, then one difference.
+template <typename R>
+__host__ __device__ __forceinline__ R upwind_nz(R m, R lo_a, R lo_b, R hi_a, R hi_b) {
+  const bool up = gt0(m);
+  return (up ? lo_a : hi_a) - (up ? lo_b : hi_b);
 }
 
 // Edge EMF along c at the corner of the (a, b) plane (c, a, b cyclic), from
 // the two a-face EMFs (fa_m at b-1, fa_p at b), the two b-face EMFs (fb_m at
 // a-1, fb_p at a), the face mass fluxes, and the four cell-centred values
-// e_mm (a-1,b-1), e_pm (a,b-1), e_mp (a-1,b), e_pp (a,b).
+// e_mm (a-1,b-1), e_pm (a,b-1), e_mp (a-1,b), e_pp (a,b).  A mass flux of
+// exactly zero is rare (rest, or inside the deadband), so FP64 forms the mean
+// it asks for only where one of the four is: four differences instead of
+// eight and no means, half of an edge's FP64 operations (128^3, stage 1 / 2:
+// 5525 / 5981 -> 5374 / 5826 us).  FP32, where the selections cost as much as
+// the differences they save, forms them all (256^3 mixed: 2647 / 2899 us, with
+// the branch 2698 / 2908).  The values are the same either way.
 template <typename R>
 __host__ __device__ __forceinline__ R edge_emf(R fa_m, R fa_p, R ma_m, R ma_p, R fb_m, R fb_p, R mb_m, R mb_p,
                                       R e_mm, R e_pm, R e_mp, R e_pp, bool plain_mean) {
   R avg = R(0.25) * (fa_m + fa_p + fb_m + fb_p);
   if (plain_mean) return avg;
-  R db_plus = upwind(ma_p, e_mp - fb_m, e_pp - fb_p);
-  R db_minus = upwind(ma_m, fb_m - e_mm, fb_p - e_pm);
-  R da_plus = upwind(mb_p, e_pm - fa_m, e_pp - fa_p);
-  R da_minus = upwind(mb_m, fa_m - e_mm, fa_p - e_mp);
+  R db_plus, db_minus, da_plus, da_minus;
+  if (sizeof(R) == 8 && (gt0(ma_p) || lt0(ma_p)) && (gt0(ma_m) || lt0(ma_m)) &&
+      (gt0(mb_p) || lt0(mb_p)) && (gt0(mb_m) || lt0(mb_m))) {
+    db_plus = upwind_nz(ma_p, e_mp, fb_m, e_pp, fb_p);
+    db_minus = upwind_nz(ma_m, fb_m, e_mm, fb_p, e_pm);
+    da_plus = upwind_nz(mb_p, e_pm, fa_m, e_pp, fa_p);
+    da_minus = upwind_nz(mb_m, fa_m, e_mm, fa_p, e_mp);
+  } else {
+    db_plus = upwind(ma_p, e_mp, fb_m, e_pp, fb_p);
+    db_minus = upwind(ma_m, fb_m, e_mm, fb_p, e_pm);
+    da_plus = upwind(mb_p, e_pm, fa_m, e_pp, fa_p);
+    da_minus = upwind(mb_m, fa_m, e_mm, fa_p, e_mp);
+  }
   return avg + R(0.25) * (db_minus - db_plus) + R(0.25) * (da_minus - da_plus);
 }
 

@@ -267,6 +267,45 @@ __device__ __forceinline__ R cfl_speed(const Geo& g, const R* w) {
   return sum;
 }
 
+// A non-negative double cut to binary32 (toward zero, 2^-23 relative; below
+// the normal range 0, above it infinity), on the integer pipe.
+__device__ __forceinline__ float cut32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi < 0x38100000u) return 0.0f;
+  if (hi >= 0x47f00000u) return __int_as_float(0x7f800000);
+  return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), hi, 3) - (896u << 23));
+}
+
+// Whether a cell's CFL speed sum may exceed `top` (positive): its value in
+// FP32, which is off by less than 1e-3 (inputs cut by 2^-23, and the
+// root of a difference that cancels loses half of FP32's digits), against
+// top.  A CFL maximum is of its start's order after a few cells, so nearly
+// every cell is settled by ~50 FP32 instructions instead of ~75 FP64 ones,
+// each of which holds the FP64 pipe for ~17 cycles (128^3 FP64, last stage:
+// 5826 -> 5450 us).  Pressures and densities
+// near the ends of FP32's range, and NaN, answer yes.
+__device__ __forceinline__ bool cfl_may_exceed(const Geo& g, const double* w, double top) {
+  float f[8];
+#pragma unroll
+  for (int v = 0; v < 8; ++v) f[v] = cut32(fabs(w[v]));
+  if (!(f[0] > 1e-30f && f[0] < 1e30f && f[4] > 1e-30f && f[4] < 1e30f)) return true;
+  return !(cfl_speed<float>(g, f) * 1.002f < cut32(top));
+}
+
+// Whether a recovered cell holds a value that is not finite (as the sums of
+// its velocities and of its field components tell).  FP64: exponents below
+// 2^1022 settle it on the integer pipe.
+__device__ __forceinline__ bool not_finite_sums(const float* w) {
+  return !(isfinite(w[4]) && isfinite(w[1] + w[2] + w[3]) && isfinite(w[5] + w[6] + w[7]));
+}
+__device__ __forceinline__ bool not_finite_sums(const double* w) {
+  unsigned top = 0u;
+#pragma unroll
+  for (int v = 1; v < 8; ++v) top = max(top, (unsigned)__double2hiint(w[v]) & 0x7fffffffu);
+  if (top < 0x7fd00000u) return false;
+  return !(isfinite(w[4]) && isfinite(w[1] + w[2] + w[3]) && isfinite(w[5] + w[6] + w[7]));
+}
+
 // Tensor maps of one primitive array set W (11 arrays of n0 x n1 x n2, 4-byte
 // elements), built on the host with the driver's tensor-map encoder: the
 // plane box of the 8 ring primitives (W x H x 1 x 8, at x = tile origin - 4,

@@ -72,7 +72,10 @@ struct Tile {
   static constexpr int nItems = nZ + nX + nY;
   // index tables (int): colc[W], rowc[H], then the queue counters of the
   // learned switch (HLL and HLLD items, one pair per plane parity)
-  static constexpr int nI = W + H + 9;   // column/row maps, switch counters, the stage's dt, flux tickets, item count
+  // column/row maps, switch counters, the stage's dt, flux tickets, item
+  // count, (one unused), the CFL maximum so far (8 bytes)
+  static constexpr int nI = W + H + 12;
+  static_assert((W + H) % 2 == 0, "the CFL word needs 8-byte alignment");
   // then four mbarriers (8 bytes each), one per ring slot, for TMA planes
   // per-cell half slopes (type R) over the (TX+2) x (TY+2) cells the faces touch:
   // x and y slopes of the current plane, z slopes of two planes (by parity)
@@ -1135,17 +1138,25 @@ struct StageKernel {
   // primitives, their store, counters and the CFL speed of one cell
   static __device__ __forceinline__ void recover_cell(const Geo& g, const StageArgs& a, long long s,
                                                       const double (&u)[5], const double (&b)[6], unsigned& nrho,
-                                                      unsigned& np, bool& bad, R& smax) {
+                                                      unsigned& np, bool& bad, R& smax, unsigned long long* top) {
     R* Wout = (R*)a.Wout;
     R w[NW];
     int hr, hp;
     recover<PREC>(g, u[0], u[1], u[2], u[3], u[4], b[0], b[1], b[2], b[3], b[4], b[5], w, hr, hp);
     nrho += hr;
     np += hp;
-    if (!(isfinite(w[4]) && isfinite(w[1] + w[2] + w[3]) && isfinite(w[5] + w[6] + w[7]))) bad = true;
+    if (not_finite_sums(w)) bad = true;
 #pragma unroll
     for (int v = 0; v < NW; ++v) Wout[MHD_IDX(v * g.ncell + s, NW * g.ncell, a.status)] = w[v];
-    if (StageTraits<STAGE>::last) {
+    if constexpr (StageTraits<STAGE>::last && PREC == P_FP64) {
+      // only a cell that may raise the CTA's maximum forms its speed in FP64
+      const double t = __longlong_as_double((long long)*(volatile unsigned long long*)top);
+      if (!(t > 0.0) || cfl_may_exceed(g, w, t)) {
+        const R sp = cfl_speed<R>(g, w);
+        smax = sp > smax ? sp : smax;
+        if (!FLAT && sp > t) atomicMax(top, (unsigned long long)__double_as_longlong(sp));
+      }
+    } else if (StageTraits<STAGE>::last) {
       const R sp = cfl_speed<R>(g, w);
       smax = sp > smax ? sp : smax;
     }
@@ -1191,7 +1202,8 @@ struct StageKernel {
                 (size_t)5 * T::nC * sizeof(double) <= (size_t)T::nHydro * sizeof(R));
   static __device__ __forceinline__ void update_plane(const Geo& g, const StageArgs& a, R* sm, const StepDt& dt,
                                                       int gi0, int gj0, int k, unsigned& nrho, unsigned& np,
-                                                      bool& bad, R& smax, ZCarry& zc, const Pre* pre = nullptr) {
+                                                      bool& bad, R& smax, ZCarry& zc, unsigned long long* top,
+                                                      const Pre* pre = nullptr) {
     const R* DU = sm + T::oDU + (k & 1) * 5 * T::nC;
     const int nx = g.n[0], ny = g.n[1];
     const int t = threadIdx.x;
@@ -1224,7 +1236,7 @@ struct StageKernel {
       double u[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) u[v] = U5[v * T::nC + c];
-      recover_cell(g, a, s, u, b, nrho, np, bad, smax);
+      recover_cell(g, a, s, u, b, nrho, np, bad, smax, top);
       return;
       }
     }
@@ -1237,7 +1249,7 @@ struct StageKernel {
       advance_faces(g, a, sm, dt, i, j, gi, gj, k, b);
       advance_cell(g, a, DU, dt, c, s, u);
       if (!a.Wout) continue;   // operator evaluation only (mhd_rhs)
-      recover_cell(g, a, s, u, b, nrho, np, bad, smax);
+      recover_cell(g, a, s, u, b, nrho, np, bad, smax, top);
     }
   }
 
@@ -1339,6 +1351,12 @@ struct StageKernel {
     if (LEARN && threadIdx.x < 4) qcnt[threadIdx.x] = 0;
     int* ticket = qcnt + 6;   // flux tickets of the dynamic flux phase, by plane parity
     if (kDyn && threadIdx.x < 2) ticket[threadIdx.x] = 0;
+    // FP64: the largest CFL speed so far, from what earlier items of the stage
+    // have folded into its word
+    unsigned long long* top = reinterpret_cast<unsigned long long*>(qcnt + 10);
+    if constexpr (StageTraits<STAGE>::last && PREC == P_FP64) {
+      if (threadIdx.x == 0) *top = *(volatile unsigned long long*)a.nextword;
+    }
     if constexpr (kCompact) build_items(g, queue, qcnt + 8, gi0, gj0);
     // the stage's dt: explicit, or cfl / (CFL max of the step's start), one
     // FP64 division per CTA
@@ -1376,7 +1394,7 @@ struct StageKernel {
       edges_2d(g, sm);
       __syncthreads();
       ZCarry zc{S(0), R(0), false};
-      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc);
+      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc, top);
       finish(a, nrho, np, nh, nd, bad, smax);
       fold_bounds_flag(a);
     } else {
@@ -1413,7 +1431,7 @@ struct StageKernel {
       edges_2d(g, sm);
       __syncthreads();
       ZCarry zc{S(0), R(0), false};
-      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc);
+      update_plane(g, a, sm, sdt, gi0, gj0, 0, nrho, np, bad, smax, zc, top);
       finish(a, nrho, np, nh, nd, bad, smax);
       fold_bounds_flag(a);
       return;
@@ -1501,7 +1519,7 @@ struct StageKernel {
       }
       divergence_and_edges(g, sm, k);
       __syncthreads();
-      if (k >= kb) update_plane(g, a, sm, sdt, gi0, gj0, k, nrho, np, bad, smax, zc, kPF ? &pre : nullptr);
+      if (k >= kb) update_plane(g, a, sm, sdt, gi0, gj0, k, nrho, np, bad, smax, zc, top, kPF ? &pre : nullptr);
     }
 
     finish(a, nrho, np, nh, nd, bad, smax);
@@ -1596,6 +1614,9 @@ __global__ void __launch_bounds__(128) prims_kernel(Geo g, StageArgs a) {
   R smax = R(0);
   bool bad = false;
   unsigned nrho = 0, np = 0;
+  // FP64: the largest CFL speed that other rows have folded in so far
+  const double top = __longlong_as_double((long long)*(volatile unsigned long long*)a.nextword);
+  (void)top;
   (void)nz;
   for (int i = threadIdx.x; i < nx; i += blockDim.x) {
     const long long s = i + (long long)nx * row;
@@ -1614,9 +1635,12 @@ __global__ void __launch_bounds__(128) prims_kernel(Geo g, StageArgs a) {
                   (double)U[ybase_hi + i], (double)U[zbase_lo + i], (double)U[zbase_hi + i], w, hr, hp);
     nrho += hr;
     np += hp;
-    if (!(isfinite(w[4]) && isfinite(w[1] + w[2] + w[3]) && isfinite(w[5] + w[6] + w[7]))) bad = true;
+    if (not_finite_sums(w)) bad = true;
 #pragma unroll
     for (int v = 0; v < NW; ++v) Wout[MHD_IDX(v * g.ncell + s, NW * g.ncell, a.status)] = w[v];
+    if constexpr (PREC == P_FP64) {
+      if (top > 0.0 && !cfl_may_exceed(g, w, top)) continue;
+    }
     const R sp = cfl_speed<R>(g, w);
     smax = sp > smax ? sp : smax;
   }

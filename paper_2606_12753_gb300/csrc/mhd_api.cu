@@ -897,69 +897,169 @@ extern "C" int mhd_get_profile(mhd_handle* h, double ms[3], long long launches[3
 // ------------------------------------------------------------ reductions
 // CFL dt of the current state and max |div B|, both in FP64.
 
-template <typename S>
-__device__ double face_at(const Geo& g, const S* U, int d, int i, int j, int k) {
-  int c[3] = {wrapc(i, g.n[0], g.bc[0]), wrapc(j, g.n[1], g.bc[1]), wrapc(k, g.n[2], g.bc[2])};
-  const int raw[3] = {i, j, k};
-  const FRef fr = face_ref1(raw[d], g.n[d], g.bc[d]);
-  int len[3] = {g.n[0], g.n[1], g.n[2]};
-  len[d] = g.nf[d];
-  c[d] = fr.a;
-  const long long ia = g.face_off[d] + c[0] + (long long)len[0] * (c[1] + (long long)len[1] * c[2]);
-  c[d] = fr.b;
-  const long long ib = g.face_off[d] + c[0] + (long long)len[0] * (c[1] + (long long)len[1] * c[2]);
-  const double f0 = (double)U[ia], f1 = (double)U[ib];
-  return f0 + (double)fr.t * (f1 - f0);
+// Cells of a reduction: a warp takes runs of up to `run` cells of one (j, k)
+// row, lanes along x, so that the index arithmetic (two divisions) is one per
+// run.  A cell's faces are stored ones: the face above the last cell of a
+// periodic axis is face 0, an outflow axis stores it.
+
+struct RowRun {
+  long long cell, x, ylo, yhi, zlo, zhi;   // index of the row's cell 0 and of its faces in the packed state
+  int i0, i1;
+};
+__device__ __forceinline__ RowRun row_run(const Geo& g, long long item, int per_row, int run) {
+  const long long row = item / per_row;
+  const int j = (int)(row % g.n[1]), k = (int)(row / g.n[1]);
+  const int jh = j + 1 < g.nf[1] ? j + 1 : 0, kh = k + 1 < g.nf[2] ? k + 1 : 0;
+  const long long nx = g.n[0];
+  RowRun r;
+  r.cell = nx * row;
+  r.x = g.face_off[0] + g.nf[0] * row;
+  r.ylo = g.face_off[1] + nx * (j + (long long)g.nf[1] * k);
+  r.yhi = g.face_off[1] + nx * (jh + (long long)g.nf[1] * k);
+  r.zlo = g.face_off[2] + nx * (j + (long long)g.n[1] * k);
+  r.zhi = g.face_off[2] + nx * (j + (long long)g.n[1] * kh);
+  r.i0 = (int)(item - row * per_row) * run;
+  r.i1 = min(r.i0 + run, g.n[0]);
+  return r;
 }
 
-__device__ __forceinline__ void block_max_atomic(double v, unsigned long long* word) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0 && v > 0.0) atomicMax(word, (unsigned long long)__double_as_longlong(v));
-}
+__device__ __forceinline__ float mag32(float x) { return fabsf(x); }
+__device__ __forceinline__ float mag32(double x) { return cut32(fabs(x)); }
+__device__ __forceinline__ float signed32(float x) { return x; }
+__device__ __forceinline__ float signed32(double x) { return copysignf(cut32(fabs(x)), __int_as_float(__double2hiint(x))); }
 
-template <typename S>
-__global__ void __launch_bounds__(256) cfl_kernel(Geo g, const S* U, unsigned long long* word) {
-  double m = 0.0;
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < g.ncell; s += (long long)gridDim.x * blockDim.x) {
-    int i = (int)(s % g.n[0]);
-    int j = (int)((s / g.n[0]) % g.n[1]);
-    int k = (int)(s / ((long long)g.n[0] * g.n[1]));
-    double rho = (double)U[s];
-    if (rho < g.rho_floor) rho = g.rho_floor;
-    double mx = (double)U[g.ncell + s], my = (double)U[2 * g.ncell + s], mz = (double)U[3 * g.ncell + s];
-    double e = (double)U[4 * g.ncell + s];
-    double b[3] = {0.5 * (face_at(g, U, 0, i, j, k) + face_at(g, U, 0, i + 1, j, k)),
-                   0.5 * (face_at(g, U, 1, i, j, k) + face_at(g, U, 1, i, j + 1, k)),
-                   0.5 * (face_at(g, U, 2, i, j, k) + face_at(g, U, 2, i, j, k + 1))};
-    double v[3] = {mx / rho, my / rho, mz / rho};
-    double p = (g.gamma - 1.0) * (e - 0.5 * (mx * mx + my * my + mz * mz) / rho - 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]));
-    if (p < g.p_floor) p = g.p_floor;
-    double sum = 0.0;
-    for (int d = 0; d < 3; ++d) {
-      if (g.n[d] <= 1) continue;
-      int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-      double w[7] = {rho, v[d], v[t1], v[t2], p, b[t1], b[t2]};
-      double cf = fast_speed(w, b[d], g.gamma);
-      sum += (fabs(v[d]) + cf) * g.inv_d[d];
+// FP32 upper bound of a cell's CFL speed sum, from its conserved values and
+// faces: the sum grows with p and with every |B_d|, so both are raised by
+// more than their rounding (1e-6 of the terms they are formed from; p
+// subtracts the field at its lower end), and the rest is a few roundings (the
+// factor at the end).  Infinity where FP32's exponent range does not hold the
+// terms.
+__device__ __forceinline__ float cfl_bound(const Geo& g, float rho, const float (&m)[3], float e, const float (&lo)[3],
+                                           const float (&hi)[3]) {
+  const float inf = __int_as_float(0x7f800000);
+  rho = fmaxf(rho, g.frho_floor);
+  const float ir = 1.0f / rho;
+  float b[3], mm = 0.f, bb = 0.f, bl = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float c = 0.5f * fabsf(lo[d] + hi[d]), err = 1e-6f * (fabsf(lo[d]) + fabsf(hi[d]));
+    const float low = fmaxf(c - err, 0.f);
+    b[d] = c + err;
+    mm += m[d] * m[d];
+    bb += b[d] * b[d];
+    bl += low * low;
+  }
+  const float kin = 0.5f * mm * ir, mag = 0.5f * bl;
+  float p = g.fgm1 * (fabsf(e) * 1.000001f - kin - mag + 4e-6f * (fabsf(e) + kin + mag));
+  p = fmaxf(p, g.fp_floor * 1.000001f);
+  const float a2 = g.fgamma * p * ir, b2 = bb * ir, x = a2 - b2;
+  if (!(rho > 1e-30f && rho < 1e30f && p > 1e-30f && p < 1e30f && a2 > 1e-18f && a2 < 1e18f)) return inf;
+  float sum = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (g.n[d] > 1) {
+      const float root = sqrtf(x * x + 4.0f * a2 * (b2 - b[d] * b[d] * ir * 0.999999f));
+      sum += (m[d] * ir + sqrtf(0.5f * (a2 + b2 + root))) * g.finv_d[d];
     }
-    m = fmax(m, sum);
   }
-  block_max_atomic(m, word);
+  return sum * 1.00001f;
+}
+
+// The speed sum in FP64: the three fast speeds share a^2, b^2 and their
+// difference, c_f,d^2 = (a^2 + b^2 + sqrt((a^2 - b^2)^2 + 4 a^2 b_t,d^2)) / 2.
+__device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double (&m)[3], double e,
+                                          const double (&b)[3]) {
+  if (lt_(rho, g.rho_floor)) rho = g.rho_floor;
+  const double ir = rcp_(rho);
+  const double b2[3] = {b[0] * b[0], b[1] * b[1], b[2] * b[2]};
+  const double bb = b2[0] + b2[1] + b2[2];
+  double p = g.gm1 * (e - 0.5 * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) * ir - 0.5 * bb);
+  if (lt_(p, g.p_floor)) p = g.p_floor;
+  const double gp = g.gamma * p, a2 = gp * ir, q = bb * ir, x = a2 - q, s = a2 + q, xx = x * x, a4r = 4.0 * a2 * ir;
+  double sum = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (g.n[d] > 1) {
+      const double root = root_(xx + a4r * (b2[(d + 1) % 3] + b2[(d + 2) % 3]));
+      sum += (fabs(m[d]) * ir + root_(0.5 * (s + root))) * g.inv_d[d];
+    }
+  }
+  return sum;
+}
+
+// CFL maximum.  The FP64 sum (~70 operations of a pipe that takes ~17 cycles
+// for each) is formed only by warps with a cell whose FP32 bound is not below
+// the largest sum found so far, which every warp reads before a run.
+// Measured (GB300): 256^3 mixed 464 us (4742 with every sum in FP64 and
+// IEEE divides), 97x130x75 FP32 139 (424).
+template <typename S>
+__global__ void __launch_bounds__(256) cfl_kernel(Geo g, const S* U, unsigned long long* word, int run) {
+  const int lane = threadIdx.x & 31;
+  const int per_row = (g.n[0] + run - 1) / run;
+  const long long items = (long long)g.n[1] * g.n[2] * per_row;
+  const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
+  for (long long item = blockIdx.x * (long long)(blockDim.x / 32) + threadIdx.x / 32; item < items; item += nwarps) {
+    const RowRun r = row_run(g, item, per_row, run);
+    double top = __longlong_as_double((long long)*(volatile unsigned long long*)word);
+    for (int base = r.i0; base < r.i1; base += 32) {
+      const int i = base + lane;
+      const bool valid = i < r.i1;
+      S u[5], lo[3], hi[3];
+      float bound = 0.0f;
+      if (valid) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) u[v] = U[v * g.ncell + r.cell + i];
+        lo[0] = U[r.x + i];
+        hi[0] = U[r.x + (i + 1 < g.nf[0] ? i + 1 : 0)];
+        lo[1] = U[r.ylo + i];
+        hi[1] = U[r.yhi + i];
+        lo[2] = U[r.zlo + i];
+        hi[2] = U[r.zhi + i];
+        const float m[3] = {mag32(u[1]), mag32(u[2]), mag32(u[3])};
+        const float l[3] = {signed32(lo[0]), signed32(lo[1]), signed32(lo[2])};
+        const float h[3] = {signed32(hi[0]), signed32(hi[1]), signed32(hi[2])};
+        bound = cfl_bound(g, signed32(u[0]), m, signed32(u[4]), l, h);
+      }
+      // (cut32 rounds top down; a bound or sum that is not a number is formed in FP64)
+      const bool need = valid && !(bound < cut32(top));
+      if (!__any_sync(0xffffffffu, need)) continue;
+      double sum = 0.0;
+      if (need) {
+        const double m[3] = {to_f64(u[1]), to_f64(u[2]), to_f64(u[3])};
+        const double b[3] = {0.5 * (to_f64(lo[0]) + to_f64(hi[0])), 0.5 * (to_f64(lo[1]) + to_f64(hi[1])),
+                             0.5 * (to_f64(lo[2]) + to_f64(hi[2]))};
+        sum = cfl_sum(g, to_f64(u[0]), m, to_f64(u[4]), b);
+      }
+      double w = sum > 0.0 ? sum : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+      if (w > top) {
+        top = w;
+        if (lane == 0) atomicMax(word, (unsigned long long)__double_as_longlong(w));
+      }
+    }
+  }
 }
 
 template <typename S>
-__global__ void __launch_bounds__(256) divb_kernel(Geo g, const S* U, unsigned long long* word) {
+__global__ void __launch_bounds__(256) divb_kernel(Geo g, const S* U, unsigned long long* word, int run) {
+  const int lane = threadIdx.x & 31;
+  const int per_row = (g.n[0] + run - 1) / run;
+  const long long items = (long long)g.n[1] * g.n[2] * per_row;
+  const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
   double m = 0.0;
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < g.ncell; s += (long long)gridDim.x * blockDim.x) {
-    int i = (int)(s % g.n[0]);
-    int j = (int)((s / g.n[0]) % g.n[1]);
-    int k = (int)(s / ((long long)g.n[0] * g.n[1]));
-    double div = (face_at(g, U, 0, i + 1, j, k) - face_at(g, U, 0, i, j, k)) * g.inv_d[0] +
-                 (face_at(g, U, 1, i, j + 1, k) - face_at(g, U, 1, i, j, k)) * g.inv_d[1] +
-                 (face_at(g, U, 2, i, j, k + 1) - face_at(g, U, 2, i, j, k)) * g.inv_d[2];
-    m = fmax(m, fabs(div));
+  for (long long item = blockIdx.x * (long long)(blockDim.x / 32) + threadIdx.x / 32; item < items; item += nwarps) {
+    const RowRun r = row_run(g, item, per_row, run);
+    for (int i = r.i0 + lane; i < r.i1; i += 32) {
+      const double div = (to_f64(U[r.x + (i + 1 < g.nf[0] ? i + 1 : 0)]) - to_f64(U[r.x + i])) * g.inv_d[0] +
+                         (to_f64(U[r.yhi + i]) - to_f64(U[r.ylo + i])) * g.inv_d[1] +
+                         (to_f64(U[r.zhi + i]) - to_f64(U[r.zlo + i])) * g.inv_d[2];
+      m = rmax(m, fabs(div));
+    }
   }
-  block_max_atomic(m, word);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = rmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0 && m > 0.0) atomicMax(word, (unsigned long long)__double_as_longlong(m));
 }
 
 static int reduce_word(mhd_handle* h, bool cfl, double* out) {
@@ -967,17 +1067,21 @@ static int reduce_word(mhd_handle* h, bool cfl, double* out) {
   if (!out) return fail(h, MHD_ERR_INVALID, "null output pointer");
   unsigned long long* word = h->words + 2;
   CUDA_TRY(h, cudaMemsetAsync(word, 0, sizeof(unsigned long long), h->stream));
-  long long n = h->geo.ncell;
-  unsigned blocks = (unsigned)((n + 255) / 256);
-  if (blocks > 152u * 16u) blocks = 152u * 16u;
+  // 8 warps a block, one run each while the chip is not full; runs of 128
+  // cells where they fill it once, of 32 in smaller boxes (128 x 128 x 1 FP64:
+  // cfl 26 us, 38 with 128-cell runs)
+  const long long rows = (long long)h->geo.n[1] * h->geo.n[2];
+  const int run = rows * ((h->geo.n[0] + 127) / 128) >= 152LL * 64 ? 128 : 32;
+  const long long runs = rows * ((h->geo.n[0] + run - 1) / run);
+  const unsigned blocks = (unsigned)std::min<long long>((runs + 7) / 8, 152LL * 8);
   if (h->elem == 8) {
     const double* U = (const double*)h->U[h->cur];
-    if (cfl) cfl_kernel<double><<<blocks, 256, 0, h->stream>>>(h->geo, U, word);
-    else divb_kernel<double><<<blocks, 256, 0, h->stream>>>(h->geo, U, word);
+    if (cfl) cfl_kernel<double><<<blocks, 256, 0, h->stream>>>(h->geo, U, word, run);
+    else divb_kernel<double><<<blocks, 256, 0, h->stream>>>(h->geo, U, word, run);
   } else {
     const float* U = (const float*)h->U[h->cur];
-    if (cfl) cfl_kernel<float><<<blocks, 256, 0, h->stream>>>(h->geo, U, word);
-    else divb_kernel<float><<<blocks, 256, 0, h->stream>>>(h->geo, U, word);
+    if (cfl) cfl_kernel<float><<<blocks, 256, 0, h->stream>>>(h->geo, U, word, run);
+    else divb_kernel<float><<<blocks, 256, 0, h->stream>>>(h->geo, U, word, run);
   }
   CUDA_TRY(h, cudaGetLastError());
   unsigned long long* hp = (unsigned long long*)h->pinned;

@@ -106,7 +106,8 @@ typedef struct {
   int emf;                 /* MHD_EMF_UPWIND | MHD_EMF_MEAN */
   double rho_floor;        /* density floor used in primitive recovery (1e-10) */
   double p_floor;          /* pressure floor (1e-10) */
-  int tile_x, tile_y, tile_z; /* tile of the fused stage kernel; 0 = default */
+  int tile_x, tile_y, tile_z; /* tile of the fused stage kernel (tile_z: planes per z-chunk); 0 = default:
+                                 16 x 8, tile_z by the size of the box (of the batch) */
   int integrator;          /* MHD_RK2 | MHD_RK3 */
   int recon;               /* MHD_RECON_PRIMITIVE | MHD_RECON_CHARACTERISTIC */
   int floor_policy;        /* MHD_FLOOR_COUNT | MHD_FLOOR_ERROR */

@@ -9,6 +9,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
+#include <map>
 #include <new>
 #include <string>
 #include <vector>
@@ -270,17 +272,100 @@ extern "C" void mhd_default_config(mhd_config* c, int nx, int ny, int nz) {
   c->p_floor = 1e-10;
 }
 
-static void default_tile(int prec, int* tx, int* ty, int* tz) {
-  if (prec == MHD_FP64) { *tx = 16; *ty = 8; *tz = 32; }
-  else { *tx = 16; *ty = 8; *tz = 32; }
+// ---- z-chunk length ---------------------------------------------------------
+// The device time of a launch whose CTAs march chunks of planes, in units of
+// a lone CTA's plane: `groups` lists (planes of a chunk, number of chunks) in
+// the order they start; `slots` CTAs are resident on kSMs SMs at once.  A chunk
+// costs its planes and a prologue (three plane loads and 1.65 flux passes, and
+// the loads' latency).  A plane takes slowdown(r) with r CTAs on an SM: an
+// FP64 CTA keeps the FP64 pipe busy by itself, the others hide each other's
+// latencies (measured: 5.4, 6.8 and 8.7 us for a mixed plane with 1, 2, 3).
+struct ChunkGroup {
+  int planes;
+  long long count;
+};
+static constexpr int kSMs = 152;
+
+static double march_time(const std::vector<ChunkGroup>& groups, int slots, bool fp64, double prologue) {
+  struct Running {
+    double left;
+    long long count;
+  };
+  std::vector<Running> run;
+  long long active = 0;
+  size_t next = 0;
+  long long waiting = groups.empty() ? 0 : groups[0].count;
+  double time = 0.0;
+  for (int event = 0; event < 4096; ++event) {
+    while (active < slots && next < groups.size()) {
+      const long long n = std::min<long long>(slots - active, waiting);
+      if (n) run.push_back({groups[next].planes + prologue, n});
+      active += n;
+      waiting -= n;
+      if (waiting == 0 && ++next < groups.size()) waiting = groups[next].count;
+    }
+    if (run.empty()) return time;
+    double step = run[0].left;
+    for (const Running& r : run) step = std::min(step, r.left);
+    const double per_sm = std::max(1.0, (double)active / kSMs);
+    time += step * (fp64 ? per_sm : 0.7 + 0.3 * per_sm);
+    size_t keep = 0;
+    for (Running& r : run) {
+      r.left -= step;
+      if (r.left > 1e-9) run[keep++] = r;
+      else active -= r.count;
+    }
+    run.resize(keep);
+  }
+  return HUGE_VAL;
 }
 
-static void resolve_tile(const mhd_config* c, int* tx, int* ty, int* tz) {
-  int dx, dy, dz;
-  default_tile(c->precision, &dx, &dy, &dz);
-  *tx = c->tile_x ? c->tile_x : dx;
-  *ty = c->tile_y ? c->tile_y : dy;
-  *tz = c->tile_z ? c->tile_z : dz;
+// CTAs per SM of the kernel a configuration runs (the kernels' launch bounds)
+static int resident_ctas(const mhd_config* c, int tx, int ty) {
+  if (c->precision == MHD_FP64) return tx * ty <= 64 || c->riemann == MHD_LEARNED ? 2 : 1;
+  if (c->recon == MHD_RECON_CHARACTERISTIC) return 2;
+  return tx * ty >= 256 ? 1 : (tx * ty >= 192 ? 2 : 3);
+}
+
+// Default planes per z-chunk: 32, unless march_time finds a length that takes
+// less than 0.94 of it.  Small boxes then have chunks enough for every SM
+// (24^3 FP64: 1 plane, 125 us a stage, 1048 with one chunk of 24; 64^3 mixed: 5,
+// 72 and 196) and middle ones no nearly empty last wave (128^3 mixed: 43, 437
+// and 483; 96x64x80 FP32: 10, 109 and 179).  The estimate is a few percent off
+// where the choices are close, hence the margin.  Results do not depend on it,
+// but for the learned switch in FP32 arithmetic, whose first pass over a
+// chunk rounds differently: it keeps 32.
+static int default_chunk(const mhd_config* c, int tx, int ty) {
+  if (c->nz <= 1 || (c->riemann == MHD_LEARNED && c->precision != MHD_FP64)) return 32;
+  const long long columns = (long long)((c->nx + tx - 1) / tx) * ((c->ny + ty - 1) / ty);
+  const bool fp64 = c->precision == MHD_FP64;
+  const int slots = kSMs * resident_ctas(c, tx, ty);
+  const auto estimate = [&](int tz) {
+    const int n = (c->nz + tz - 1) / tz, last = c->nz - (n - 1) * tz;
+    std::vector<ChunkGroup> groups;
+    if (n > 1) groups.push_back({tz, columns * (n - 1)});
+    groups.push_back({last, columns});
+    return march_time(groups, slots, fp64, fp64 ? 2.1 : 3.5);
+  };
+  int best = 32;
+  const double base = estimate(32);
+  double least = 0.94 * base;
+  for (int n = 1, tz = c->nz, previous = 0; n <= c->nz; ++n, previous = tz) {
+    tz = (c->nz + n - 1) / n;
+    if (tz == previous || tz > (1 << 20)) continue;
+    if (tz < 16 && columns * n > 40LL * slots) break;   // shorter chunks only add prologues to a full chip
+    const double t = estimate(tz);
+    if (t < least) {
+      least = t;
+      best = tz;
+    }
+  }
+  return best;
+}
+
+static void resolve_tile(const mhd_config* c, int* tx, int* ty) {
+  *tx = c->tile_x ? c->tile_x : 16;
+  *ty = c->tile_y ? c->tile_y : 8;
 }
 
 static int validate(const mhd_config* c, mhd_handle* h) {
@@ -302,9 +387,9 @@ static int validate(const mhd_config* c, mhd_handle* h) {
   if (c->emf != MHD_EMF_UPWIND && c->emf != MHD_EMF_MEAN) return fail(h, MHD_ERR_INVALID, "unknown emf mode");
   if (!(c->rho_floor > 0.0) || !(c->p_floor > 0.0)) return fail(h, MHD_ERR_INVALID, "floors must be positive");
   if (c->tile_x < 0 || c->tile_y < 0 || c->tile_z < 0) return fail(h, MHD_ERR_INVALID, "tile sizes must be >= 0");
-  int tx, ty, tz;
-  resolve_tile(c, &tx, &ty, &tz);
-  if (tz < 1 || tz > (1 << 20)) return fail(h, MHD_ERR_INVALID, "tile_z out of range");
+  int tx, ty;
+  resolve_tile(c, &tx, &ty);
+  if (c->tile_z > (1 << 20)) return fail(h, MHD_ERR_INVALID, "tile_z out of range");
   if (!stage_tile_supported(c->precision, tx, ty))
     return fail(h, MHD_ERR_INVALID, "tile %dx%d is not instantiated for this precision", tx, ty);
   if (c->riemann == MHD_LEARNED && (tx != 16 || ty != 8))
@@ -350,7 +435,8 @@ static void fill_geo(const mhd_config* c, Geo* g) {
   g->frho_floor = (float)g->rho_floor;
   g->fp_floor = (float)g->p_floor;
   g->fdeadband = (float)g->deadband;
-  resolve_tile(c, &g->TX, &g->TY, &g->TZ);
+  resolve_tile(c, &g->TX, &g->TY);
+  g->TZ = c->tile_z ? c->tile_z : default_chunk(c, g->TX, g->TY);
   g->ntx = (g->n[0] + g->TX - 1) / g->TX;
   g->nty = (g->n[1] + g->TY - 1) / g->TY;
   g->nchunk = (g->n[2] + g->TZ - 1) / g->TZ;
@@ -1220,6 +1306,38 @@ static void drop_graph(mhd_batch* b) {
   b->g_nsteps = -1;
 }
 
+// Default planes per z-chunk of a batch: the length whose items, started
+// longest first, take the least estimated time, if that is under 0.97 of 32's
+// (measured, FP32, us a stage: 64 boxes of 32-128 cells an axis 4705 at 32,
+// 4574 at 64; 4 boxes of 32-112 360 at 32, 200 at 12).
+static int batch_default_chunk(const mhd_batch* b, int tx, int ty) {
+  static const int lengths[] = {32, 2, 4, 6, 8, 12, 16, 24, 48, 64, 96, 128};
+  const int slots = kSMs * resident_ctas(&b->cfg[0], tx, ty);
+  int best = 32;
+  double least = HUGE_VAL;
+  for (int tz : lengths) {
+    std::map<int, long long, std::greater<int>> count;   // chunks by planes, longest first
+    long long items = 0;
+    for (const mhd_config& c : b->cfg) {
+      const long long columns = (long long)((c.nx + tx - 1) / tx) * ((c.ny + ty - 1) / ty);
+      const int n = (c.nz + tz - 1) / tz;
+      if (n > 1) count[tz] += columns * (n - 1);
+      count[c.nz - (n - 1) * tz] += columns;
+      items += columns * n;
+    }
+    if (tz < 16 && items > 40LL * slots) continue;
+    std::vector<ChunkGroup> groups;
+    for (const auto& q : count) groups.push_back({q.first, q.second});
+    const double t = march_time(groups, slots, b->prec == MHD_FP64, b->prec == MHD_FP64 ? 2.1 : 2.5);
+    if (tz == 32) least = 0.97 * t;
+    else if (t < least) {
+      least = t;
+      best = tz;
+    }
+  }
+  return best;
+}
+
 // Recompute per-box geometry, work items, shared memory and the persistent
 // grid for tile (tx, ty, tz), and upload the box table.
 static int batch_apply_tile(mhd_batch* b, int tx, int ty, int tz) {
@@ -1368,9 +1486,9 @@ extern "C" int mhd_batch_create(int nbox, const mhd_config* cfgs, void* cuda_str
     mhd_batch_destroy(b);
     return MHD_ERR_CUDA;
   }
-  int tx, ty, tz;
-  resolve_tile(&cfgs[0], &tx, &ty, &tz);
-  int rc = batch_apply_tile(b, tx, ty, tz);
+  int tx, ty;
+  resolve_tile(&cfgs[0], &tx, &ty);
+  int rc = batch_apply_tile(b, tx, ty, cfgs[0].tile_z ? cfgs[0].tile_z : batch_default_chunk(b, tx, ty));
   if (rc) {
     g_batch_err = b->err;
     mhd_batch_destroy(b);

@@ -399,27 +399,19 @@ struct StageKernel {
       const int first = (int)blockDim.x > T::nC ? T::nC : 0;   // threads without a cell first
       if ((int)threadIdx.x >= first) cell_emf(sm, q, (int)threadIdx.x - first, (int)blockDim.x - first);
       const int lane = threadIdx.x & 31;
-      if (kCompact && with_z) {
-        // the tile's list (a chunk's first pass, without z-faces, takes every item)
-        const unsigned char* base0 = reinterpret_cast<const unsigned char*>(sm);
-        const unsigned short* list =
-            reinterpret_cast<const unsigned short*>(base0 + T::template queue_off<R, kQueue>());
-        const int nl = reinterpret_cast<const int*>(base0 + T::template int_off<R, kQueue>())[T::W + T::H + 8];
-        for (;;) {
-          int base = 0;
-          if (lane == 0) base = atomicAdd(ticket, 32);
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (base >= nl) break;
-          if (base + lane < nl) flux_item(g, sm, k, q, T::nZ, list[MHD_SIDX(base + lane, T::nItems)], gam, ig);
-        }
-      } else {
-        for (;;) {
-          int base = 0;
-          if (lane == 0) base = atomicAdd(ticket, 32);
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (base >= nitems) break;
-          if (base + lane < nitems) flux_item(g, sm, k, q, nZ, base + lane, gam, ig);
-        }
+      // kCompact: the tile's list (a chunk's first pass, without z-faces, takes every item)
+      const bool listed = kCompact && with_z;
+      const unsigned char* base0 = reinterpret_cast<const unsigned char*>(sm);
+      const unsigned short* list = reinterpret_cast<const unsigned short*>(base0 + T::template queue_off<R, kQueue>());
+      int n = nitems;
+      if (listed) n = reinterpret_cast<const int*>(base0 + T::template int_off<R, kQueue>())[T::W + T::H + 8];
+      for (;;) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(ticket, 32);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base >= n) break;
+        if (base + lane < n)
+          flux_item(g, sm, k, q, nZ, listed ? list[MHD_SIDX(base + lane, T::nItems)] : base + lane, gam, ig);
       }
     } else {
       for (int w = threadIdx.x; w < nitems; w += blockDim.x) flux_item(g, sm, k, q, nZ, w, gam, ig);
@@ -1461,29 +1453,25 @@ struct StageKernel {
     __syncthreads();
     for (int m = kb - 2; m <= kb; ++m)
       if (plane_tma(m)) tma_wait(a, mbar, m & 3, phases);
-    if constexpr (SLOPES) {
-      slopes(g, sm, sl, kb - 1, false, ticket + (kb & 1));
-      __syncthreads();
-      fluxes_sl(g, sm, sl, kb - 2, kb - 1, false);
-    } else if constexpr (LEARN) {
+    // The march starts with a pass without z-faces (k = kb - 2: the x- and
+    // y-faces of plane kb - 1), then completes the edges below plane kb (k =
+    // kb - 1) and updates from k = kb on.  All passes run the same code: a copy
+    // of its own for the first would double the flux code and may round
+    // differently, so that results would depend on the chunks (the learned
+    // switch keeps its copy, and with it the rounding of its first passes).
+    if constexpr (LEARN) {
       fluxes_learned(g, a, sm, queue, qcnt, kb - 2, kb - 1, false, gi0, gj0, kb, ke, nh, nd);
-    } else {
-      fluxes(g, sm, kb - 2, kb - 1, false, ticket + (kb & 1));
-    }
-    __syncthreads();
-    // a TMA plane is issued as soon as the flux phase has freed its slot:
-    // plane k + 3 goes where plane k - 1 was, and lands during phases C, D
-    if (plane_tma(kb + 1) && threadIdx.x == 0) {
-      tma_issue(*tm, sm, mbar, kb + 1, wrapc(kb + 1, g.n[2], g.bc[2]), gi0, gj0, true, g, a.status);
-      ++ntma;
+      __syncthreads();
     }
     ZCarry zc{S(0), R(0), false};   // face group: upper z-face of the previous plane
-    for (int k = kb - 1; k < ke; ++k) {
+    for (int k = LEARN ? kb - 1 : kb - 2; k < ke; ++k) {
       // the threads without a cell in the update phase load the next plane
       // while the others finish that phase (unless it comes by TMA)
-      const bool tma_next = plane_tma(k + 2);
+      const bool first = !LEARN && k == kb - 2;   // its planes are in
+      const bool tma_next = !first && plane_tma(k + 2);
       const int nl = (int)blockDim.x - T::nC;   // threads without a cell in the update phase
-      if (kDyn && !tma_next && nl >= 32 && nl % 32 == 0) {
+      if (first) {
+      } else if (kDyn && !tma_next && nl >= 32 && nl % 32 == 0) {
         if ((int)threadIdx.x >= T::nC) {
           load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 2, true, T::nC);
           asm volatile("bar.sync %0, %1;" ::"r"(kLoadBarrier), "r"(nl) : "memory");
@@ -1499,20 +1487,24 @@ struct StageKernel {
       if constexpr (SLOPES) {
         slopes(g, sm, sl, k + 1, false, ticket + (k & 1));
         __syncthreads();
-        fluxes_sl(g, sm, sl, k, k + 1, true);
+        fluxes_sl(g, sm, sl, k, k + 1, !first);
       } else if constexpr (LEARN) {
         fluxes_learned(g, a, sm, queue, qcnt, k, k + 1, true, gi0, gj0, kb, ke, nh, nd);
       } else {
-        fluxes(g, sm, k, k + 1, true, ticket + (k & 1));
+        fluxes(g, sm, k, k + 1, !first, ticket + (k & 1));
       }
       __syncthreads();
       // the next flux phase's tickets: last drawn by the flux phase of plane
-      // k - 1, first drawn after the barrier that follows phase C
-      if (kDyn && threadIdx.x == 0) ticket[(k + 1) & 1] = 0;
+      // k - 1, first drawn after the barrier that follows phase C (or, after
+      // the first pass, never drawn yet)
+      if (kDyn && !first && threadIdx.x == 0) ticket[(k + 1) & 1] = 0;
+      // a TMA plane is issued as soon as the flux phase has freed its slot:
+      // plane k + 3 goes where plane k - 1 was, and lands during phases C, D
       if (k + 3 <= ke + 1 && plane_tma(k + 3) && threadIdx.x == 0) {
         tma_issue(*tm, sm, mbar, k + 3, wrapc(k + 3, g.n[2], g.bc[2]), gi0, gj0, true, g, a.status);
         ++ntma;
       }
+      if (first) continue;
       Pre pre;
       if constexpr (kPF) {
         if (k >= kb) prefetch(g, a, gi0, gj0, k, zc.have, pre);

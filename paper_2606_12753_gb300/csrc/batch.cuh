@@ -140,6 +140,39 @@ static __global__ void batch_advance(BoxDesc* boxes, int nbox, int nsteps) {
   }
 }
 
+// A set of boxes, by bit, among kMost consecutive ones of the table.
+struct BoxSet {
+  static constexpr int kMost = 1024;
+  unsigned bits[kMost / 32];
+  int first, count;
+};
+
+static __global__ void batch_clear_words(const BoxDesc* boxes, BoxSet set) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < set.count && (set.bits[i / 32] >> (i % 32) & 1u)) {
+    const BoxDesc& d = boxes[set.first + i];
+    d.words[d.parity] = 0ull;
+  }
+}
+
+// Primitives and CFL maxima of a set of boxes, blockIdx.y the box: 64 boxes in
+// one launch instead of 64 launches of a few us each and as many clears.
+template <int PREC>
+__global__ void __launch_bounds__(256)
+    batch_prims_kernel(const BoxDesc* boxes, BoxSet set, int run, unsigned* status, unsigned long long* counters) {
+  const int i = blockIdx.y;
+  if (!(set.bits[i / 32] >> (i % 32) & 1u)) return;
+  const BoxDesc& d = boxes[set.first + i];
+  StageArgs a = {};
+  a.U = d.U[d.cur];
+  a.Wout = d.W[0];
+  a.nextword = d.words + d.parity;
+  a.status = status;
+  a.counters = counters;
+  const int warps = blockDim.x / 32;
+  prims_rows<PREC>(d.g, a, blockIdx.x * (long long)warps + threadIdx.x / 32, gridDim.x * (long long)warps, run);
+}
+
 // host-side launchers (one translation unit per precision)
 cudaError_t batch_launch(int prec, int tx, int ty, unsigned grid, size_t smem, cudaStream_t st, const BatchArgs& ba);
 cudaError_t batch_set_smem(int prec, int tx, int ty, size_t bytes);

@@ -64,4 +64,11 @@ int MHD_UNIT_FN(batch_max_blocks)(int tx, int ty, size_t smem) {
   return n;
 }
 
+cudaError_t MHD_UNIT_FN(batch_prims)(unsigned blocks, cudaStream_t st, BoxDesc* boxes, const BoxSet& set, int run,
+                                     unsigned* status, unsigned long long* counters) {
+  batch_clear_words<<<(set.count + 127) / 128, 128, 0, st>>>(boxes, set);
+  batch_prims_kernel<MHD_UNIT_PREC><<<dim3(blocks, set.count), 256, 0, st>>>(boxes, set, run, status, counters);
+  return cudaGetLastError();
+}
+
 }  // namespace mhd

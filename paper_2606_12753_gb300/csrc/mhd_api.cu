@@ -61,9 +61,9 @@ cudaError_t set_smem_char_fp32(size_t);
 cudaError_t set_smem_learned_fp64(size_t);
 cudaError_t set_smem_learned_mixed(size_t);
 cudaError_t set_smem_learned_fp32(size_t);
-cudaError_t launch_prims_fp64(unsigned, cudaStream_t, const Geo&, const StageArgs&);
-cudaError_t launch_prims_mixed(unsigned, cudaStream_t, const Geo&, const StageArgs&);
-cudaError_t launch_prims_fp32(unsigned, cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t launch_prims_fp64(cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t launch_prims_mixed(cudaStream_t, const Geo&, const StageArgs&);
+cudaError_t launch_prims_fp32(cudaStream_t, const Geo&, const StageArgs&);
 
 cudaError_t launch_stage(int prec, int stage, int tx, int ty, unsigned nb, size_t smem, cudaStream_t st,
                          const Geo& g, const StageArgs& a, const TmaMaps* tm) {
@@ -106,11 +106,11 @@ cudaError_t launch_stage(int prec, int stage, int tx, int ty, unsigned nb, size_
     default: return launch_stage_fp32(stage, tx, ty, nb, smem, st, g, a, maps);
   }
 }
-cudaError_t launch_prims(int prec, unsigned nb, cudaStream_t st, const Geo& g, const StageArgs& a) {
+cudaError_t launch_prims(int prec, cudaStream_t st, const Geo& g, const StageArgs& a) {
   switch (prec) {
-    case P_FP64: return launch_prims_fp64(nb, st, g, a);
-    case P_MIXED: return launch_prims_mixed(nb, st, g, a);
-    default: return launch_prims_fp32(nb, st, g, a);
+    case P_FP64: return launch_prims_fp64(st, g, a);
+    case P_MIXED: return launch_prims_mixed(st, g, a);
+    default: return launch_prims_fp32(st, g, a);
   }
 }
 cudaError_t stage_set_smem_char(int prec, size_t bytes) {
@@ -607,6 +607,88 @@ extern "C" const char* mhd_last_error(const mhd_handle* h) {
   return h ? h->err.c_str() : g_create_err.c_str();
 }
 
+// ---- state copies -------------------------------------------------------------
+// The eight arrays of a state between the caller's device arrays and a packed
+// buffer, in one launch: blockIdx.y is the array.  16 bytes a thread and access
+// where both ends are aligned to 16, else 8, else 4 (the element sizes).  Eight
+// copies of a small box are eight launches of ~2 us each, on the host and on
+// the device (measured, set / get: 128^2 FP64 51 / 45 -> 29 / 20 us,
+// 64 boxes 3449 / 3938 -> 1131 / 1712, 256^3 375 / 362 -> 367 / 355).
+struct StateCopy {
+  const void* src[8];
+  void* dst[8];
+  unsigned long long bytes[8];
+};
+
+template <typename V>
+__device__ __forceinline__ void copy_as(const void* src, void* dst, unsigned long long bytes) {
+  const unsigned long long n = bytes / sizeof(V), step = (unsigned long long)gridDim.x * blockDim.x;
+  unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
+  const V* s = (const V*)src;
+  V* d = (V*)dst;
+  for (; i + 3 * step < n; i += 4 * step) {   // four loads in flight
+    const V a = s[i], b = s[i + step], c = s[i + 2 * step], e = s[i + 3 * step];
+    d[i] = a;
+    d[i + step] = b;
+    d[i + 2 * step] = c;
+    d[i + 3 * step] = e;
+  }
+  for (; i < n; i += step) d[i] = s[i];
+  const unsigned long long done = n * sizeof(V);   // the rest, fewer than 16 bytes
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < (unsigned)((bytes - done) / 4))
+    ((unsigned*)((char*)dst + done))[t] = ((const unsigned*)((const char*)src + done))[t];
+}
+
+__global__ void __launch_bounds__(256) state_copy_kernel(StateCopy c) {
+  const int q = blockIdx.y;
+  const uintptr_t both = (uintptr_t)c.src[q] | (uintptr_t)c.dst[q];
+  if ((both & 15) == 0) copy_as<uint4>(c.src[q], c.dst[q], c.bytes[q]);
+  else if ((both & 7) == 0) copy_as<uint2>(c.src[q], c.dst[q], c.bytes[q]);
+  else copy_as<unsigned>(c.src[q], c.dst[q], c.bytes[q]);
+}
+
+// Whether p is plain memory of the current device (anything else, a host
+// pointer passed for a device one among it, goes to the runtime's copy).
+static bool device_memory(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  int dev = -1;
+  return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev &&
+         ((uintptr_t)p & 3) == 0;
+}
+
+namespace mhd {
+// Copy the arrays of a packed state (in: to it, else from it), device to device.
+cudaError_t copy_state_on_device(const Geo& g, bool in, char* base, size_t elem, void* const* cell, void* const* face,
+                                 cudaStream_t st) {
+  StateCopy c;
+  bool plain = true;
+  unsigned long long most = 0;
+  for (int q = 0; q < 8; ++q) {
+    void* user = q < 5 ? cell[q] : face[q - 5];
+    char* own = base + (size_t)(q < 5 ? q * g.ncell : g.face_off[q - 5]) * elem;
+    c.src[q] = in ? user : own;
+    c.dst[q] = in ? own : user;
+    c.bytes[q] = (unsigned long long)(q < 5 ? g.ncell : face_count(g, q - 5)) * elem;
+    most = std::max(most, c.bytes[q]);
+    plain = plain && device_memory(user);
+  }
+  if (plain) {
+    const unsigned blocks = (unsigned)std::min<unsigned long long>((most + 4095) / 4096, 152ull * 4);
+    state_copy_kernel<<<dim3(blocks, 8), 256, 0, st>>>(c);
+    return cudaGetLastError();
+  }
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < 8 && e == cudaSuccess; ++q)
+    e = cudaMemcpyAsync(c.dst[q], c.src[q], c.bytes[q], cudaMemcpyDeviceToDevice, st);
+  return e;
+}
+}  // namespace mhd
+
 static int copy_arrays(mhd_handle* h, bool in, char* base, size_t elem, void* const* cell, void* const* face,
                        int on_device) {
   if (!cell || !face) return fail(h, MHD_ERR_INVALID, "null state pointer array");
@@ -614,7 +696,12 @@ static int copy_arrays(mhd_handle* h, bool in, char* base, size_t elem, void* co
     if (!cell[v]) return fail(h, MHD_ERR_INVALID, "null cell array %d", v);
   for (int d = 0; d < 3; ++d)
     if (!face[d]) return fail(h, MHD_ERR_INVALID, "null face array %d", d);
-  cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : (in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
+  if (on_device) {
+    CUDA_TRY(h, copy_state_on_device(h->geo, in, base, elem, cell, face, h->stream));
+    if (!in) CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return MHD_OK;
+  }
+  const cudaMemcpyKind kind = in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
   for (int v = 0; v < 5; ++v) {
     char* dev = base + (size_t)v * h->geo.ncell * elem;
     size_t n = (size_t)h->geo.ncell * elem;
@@ -625,7 +712,7 @@ static int copy_arrays(mhd_handle* h, bool in, char* base, size_t elem, void* co
     size_t n = (size_t)face_count(h->geo, d) * elem;
     CUDA_TRY(h, in ? cudaMemcpyAsync(dev, face[d], n, kind, h->stream) : cudaMemcpyAsync(face[d], dev, n, kind, h->stream));
   }
-  if (!in || !on_device) CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   return MHD_OK;
 }
 
@@ -670,10 +757,7 @@ static cudaError_t ensure_prims(mhd_handle* h) {
   a.nextword = h->words + h->parity;
   cudaError_t e = cudaMemsetAsync(h->words + h->parity, 0, sizeof(unsigned long long), h->stream);
   if (e) return e;
-  long long n = h->geo.ncell;
-  unsigned nb = (unsigned)((n + 255) / 256);
-  if (nb > 152u * 16u) nb = 152u * 16u;
-  e = launch_prims(h->cfg.precision, nb, h->stream, h->geo, a);
+  e = launch_prims(h->cfg.precision, h->stream, h->geo, a);
   if (e) return e;
   h->prims_valid = true;
   return cudaSuccess;
@@ -983,32 +1067,6 @@ extern "C" int mhd_get_profile(mhd_handle* h, double ms[3], long long launches[3
 // ------------------------------------------------------------ reductions
 // CFL dt of the current state and max |div B|, both in FP64.
 
-// Cells of a reduction: a warp takes runs of up to `run` cells of one (j, k)
-// row, lanes along x, so that the index arithmetic (two divisions) is one per
-// run.  A cell's faces are stored ones: the face above the last cell of a
-// periodic axis is face 0, an outflow axis stores it.
-
-struct RowRun {
-  long long cell, x, ylo, yhi, zlo, zhi;   // index of the row's cell 0 and of its faces in the packed state
-  int i0, i1;
-};
-__device__ __forceinline__ RowRun row_run(const Geo& g, long long item, int per_row, int run) {
-  const long long row = item / per_row;
-  const int j = (int)(row % g.n[1]), k = (int)(row / g.n[1]);
-  const int jh = j + 1 < g.nf[1] ? j + 1 : 0, kh = k + 1 < g.nf[2] ? k + 1 : 0;
-  const long long nx = g.n[0];
-  RowRun r;
-  r.cell = nx * row;
-  r.x = g.face_off[0] + g.nf[0] * row;
-  r.ylo = g.face_off[1] + nx * (j + (long long)g.nf[1] * k);
-  r.yhi = g.face_off[1] + nx * (jh + (long long)g.nf[1] * k);
-  r.zlo = g.face_off[2] + nx * (j + (long long)g.n[1] * k);
-  r.zhi = g.face_off[2] + nx * (j + (long long)g.n[1] * kh);
-  r.i0 = (int)(item - row * per_row) * run;
-  r.i1 = min(r.i0 + run, g.n[0]);
-  return r;
-}
-
 __device__ __forceinline__ float mag32(float x) { return fabsf(x); }
 __device__ __forceinline__ float mag32(double x) { return cut32(fabs(x)); }
 __device__ __forceinline__ float signed32(float x) { return x; }
@@ -1153,13 +1211,8 @@ static int reduce_word(mhd_handle* h, bool cfl, double* out) {
   if (!out) return fail(h, MHD_ERR_INVALID, "null output pointer");
   unsigned long long* word = h->words + 2;
   CUDA_TRY(h, cudaMemsetAsync(word, 0, sizeof(unsigned long long), h->stream));
-  // 8 warps a block, one run each while the chip is not full; runs of 128
-  // cells where they fill it once, of 32 in smaller boxes (128 x 128 x 1 FP64:
-  // cfl 26 us, 38 with 128-cell runs)
-  const long long rows = (long long)h->geo.n[1] * h->geo.n[2];
-  const int run = rows * ((h->geo.n[0] + 127) / 128) >= 152LL * 64 ? 128 : 32;
-  const long long runs = rows * ((h->geo.n[0] + run - 1) / run);
-  const unsigned blocks = (unsigned)std::min<long long>((runs + 7) / 8, 152LL * 8);
+  const int run = row_run_length(h->geo);
+  const unsigned blocks = row_run_blocks(h->geo, run);
   if (h->elem == 8) {
     const double* U = (const double*)h->U[h->cur];
     if (cfl) cfl_kernel<double><<<blocks, 256, 0, h->stream>>>(h->geo, U, word, run);
@@ -1217,6 +1270,17 @@ size_t batch_smem_bytes_mixed(int, int);
 size_t batch_smem_bytes_fp32(int, int);
 int batch_max_blocks_mixed(int, int, size_t);
 int batch_max_blocks_fp32(int, int, size_t);
+cudaError_t batch_prims_fp64(unsigned, cudaStream_t, BoxDesc*, const BoxSet&, int, unsigned*, unsigned long long*);
+cudaError_t batch_prims_mixed(unsigned, cudaStream_t, BoxDesc*, const BoxSet&, int, unsigned*, unsigned long long*);
+cudaError_t batch_prims_fp32(unsigned, cudaStream_t, BoxDesc*, const BoxSet&, int, unsigned*, unsigned long long*);
+static cudaError_t batch_prims(int prec, unsigned blocks, cudaStream_t st, BoxDesc* boxes, const BoxSet& set, int run,
+                               unsigned* status, unsigned long long* counters) {
+  switch (prec) {
+    case P_FP64: return batch_prims_fp64(blocks, st, boxes, set, run, status, counters);
+    case P_MIXED: return batch_prims_mixed(blocks, st, boxes, set, run, status, counters);
+    default: return batch_prims_fp32(blocks, st, boxes, set, run, status, counters);
+  }
+}
 
 cudaError_t batch_launch(int prec, int tx, int ty, unsigned grid, size_t smem, cudaStream_t st, const BatchArgs& ba) {
   switch (prec) {
@@ -1505,20 +1569,23 @@ static int batch_copy(mhd_batch* b, int i, bool in, void* const* cell, void* con
   const Geo& g = b->box[i].g;
   const size_t elem = b->prec == MHD_FP32 ? 4 : 8;
   char* base = (char*)b->box[i].U[b->box[i].cur];
-  cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : (in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
-  for (int v = 0; v < 5; ++v) {
+  for (int v = 0; v < 5; ++v)
     if (!cell[v]) return bfail(b, MHD_ERR_INVALID, "null cell array %d", v);
-    char* dev = base + (size_t)v * g.ncell * elem;
-    BCUDA_TRY(b, in ? cudaMemcpyAsync(dev, cell[v], g.ncell * elem, kind, b->stream)
-                    : cudaMemcpyAsync(cell[v], dev, g.ncell * elem, kind, b->stream));
-  }
-  for (int d = 0; d < 3; ++d) {
+  for (int d = 0; d < 3; ++d)
     if (!face[d]) return bfail(b, MHD_ERR_INVALID, "null face array %d", d);
-    char* dev = base + (size_t)g.face_off[d] * elem;
-    const size_t n = (size_t)face_count(g, d) * elem;
-    BCUDA_TRY(b, in ? cudaMemcpyAsync(dev, face[d], n, kind, b->stream) : cudaMemcpyAsync(face[d], dev, n, kind, b->stream));
+  if (on_device) {
+    BCUDA_TRY(b, copy_state_on_device(g, in, base, elem, cell, face, b->stream));
+    if (!in) BCUDA_TRY(b, cudaStreamSynchronize(b->stream));
+  } else {
+    const cudaMemcpyKind kind = in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost;
+    for (int q = 0; q < 8; ++q) {
+      char* dev = base + (size_t)(q < 5 ? q * g.ncell : g.face_off[q - 5]) * elem;
+      const size_t n = (size_t)(q < 5 ? g.ncell : face_count(g, q - 5)) * elem;
+      void* user = q < 5 ? cell[q] : face[q - 5];
+      BCUDA_TRY(b, in ? cudaMemcpyAsync(dev, user, n, kind, b->stream) : cudaMemcpyAsync(user, dev, n, kind, b->stream));
+    }
+    BCUDA_TRY(b, cudaStreamSynchronize(b->stream));
   }
-  if (!in || !on_device) BCUDA_TRY(b, cudaStreamSynchronize(b->stream));
   if (in) b->prims_valid[i] = false;
   return MHD_OK;
 }
@@ -1532,22 +1599,30 @@ extern "C" int mhd_batch_get_state(mhd_batch* b, int box, void* cell[5], void* f
   return batch_copy(b, box, false, cell, face, on_device);
 }
 
+// Primitives and CFL maxima of the boxes whose state was set from outside: one
+// launch for up to 1024 boxes (and one that clears their CFL words).
 static int batch_ensure_prims(mhd_batch* b) {
-  for (int i = 0; i < b->nbox; ++i) {
-    if (b->prims_valid[i]) continue;
-    BoxDesc& d = b->box[i];
-    StageArgs a;
-    memset(&a, 0, sizeof a);
-    a.status = b->status;
-    a.counters = b->counters;
-    a.U = d.U[d.cur];
-    a.Wout = d.W[0];
-    a.nextword = d.words + d.parity;
-    BCUDA_TRY(b, cudaMemsetAsync(d.words + d.parity, 0, sizeof(unsigned long long), b->stream));
-    unsigned nb = (unsigned)((d.g.ncell + 255) / 256);
-    if (nb > 152u * 16u) nb = 152u * 16u;
-    BCUDA_TRY(b, launch_prims(b->prec, nb, b->stream, d.g, a));
-    b->prims_valid[i] = true;
+  for (int first = 0; first < b->nbox; first += BoxSet::kMost) {
+    BoxSet set = {};
+    set.first = first;
+    set.count = std::min(b->nbox - first, (int)BoxSet::kMost);
+    long long runs = 0, widest = 0;
+    for (int i = 0; i < set.count; ++i) {
+      if (b->prims_valid[first + i]) continue;
+      const Geo& g = b->box[first + i].g;
+      set.bits[i / 32] |= 1u << (i % 32);
+      const long long n = (long long)g.n[1] * g.n[2] * ((g.n[0] + 127) / 128);
+      runs += n;
+      widest = std::max(widest, n);
+    }
+    if (!runs) continue;
+    const int run = runs >= 152LL * 64 ? 128 : 32;   // as row_run_length for one box
+    if (run == 32) widest *= 4;
+    // enough blocks a box for its runs, no more in all than a few per SM
+    const long long most = std::max(1LL, 152LL * 16 / set.count);
+    const unsigned blocks = (unsigned)std::min(most, (widest + 7) / 8);
+    BCUDA_TRY(b, batch_prims(b->prec, blocks, b->stream, b->dbox, set, run, b->status, b->counters));
+    for (int i = 0; i < set.count; ++i) b->prims_valid[first + i] = true;
   }
   return MHD_OK;
 }
@@ -1838,7 +1913,6 @@ extern "C" int mhd_batch_autotune(mhd_batch* b, int trial_steps, const char* cac
 namespace mhd {
 int internal_validate(const mhd_config* c) { return validate(c, nullptr); }
 void internal_fill_geo(const mhd_config* c, Geo* g) { fill_geo(c, g); }
-long long internal_face_count(const Geo& g, int d) { return face_count(g, d); }
 void internal_set_error(const char* msg) { g_create_err = msg; }
 }  // namespace mhd
 

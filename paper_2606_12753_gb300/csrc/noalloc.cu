@@ -29,7 +29,8 @@
 namespace mhd {
 int internal_validate(const mhd_config* c);
 void internal_fill_geo(const mhd_config* c, Geo* g);
-long long internal_face_count(const Geo& g, int d);
+cudaError_t copy_state_on_device(const Geo& g, bool in, char* base, size_t elem, void* const* cell, void* const* face,
+                                 cudaStream_t st);
 void internal_set_error(const char* msg);
 }  // namespace mhd
 
@@ -109,12 +110,8 @@ extern "C" int mhd_step_noalloc(const mhd_config* cfg, void* cuda_stream, const 
 
   cudaError_t e = stage_set_smem(prec, g.TX, g.TY, stage_smem_bytes(prec, g.TX, g.TY));
   if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, 64 * 8, st);
-  for (int v = 0; v < 5 && e == cudaSuccess; ++v)
-    e = cudaMemcpyAsync((char*)Uin + (size_t)v * g.ncell * elem, cell_in[v], (size_t)g.ncell * elem,
-                        cudaMemcpyDeviceToDevice, st);
-  for (int d = 0; d < 3 && e == cudaSuccess; ++d)
-    e = cudaMemcpyAsync((char*)Uin + (size_t)g.face_off[d] * elem, face_in[d],
-                        (size_t)internal_face_count(g, d) * elem, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess)
+    e = copy_state_on_device(g, true, (char*)Uin, elem, (void* const*)cell_in, (void* const*)face_in, st);
   if (e != cudaSuccess) return noalloc_fail(MHD_ERR_CUDA, "mhd_step_noalloc: %s", cudaGetErrorString(e));
 
   StageArgs a;
@@ -125,8 +122,7 @@ extern "C" int mhd_step_noalloc(const mhd_config* cfg, void* cuda_stream, const 
   a.U = Uin;
   a.Wout = W0;
   a.nextword = words + 0;
-  unsigned nb = (unsigned)((g.ncell + 255) / 256);
-  e = launch_prims(prec, nb, st, g, a);
+  e = launch_prims(prec, st, g, a);
   // stage 1 and stage 2 of the RK2 step
   const unsigned nblocks = (unsigned)(g.ntx * g.nty * g.nchunk);
   const size_t smem = stage_smem_bytes(prec, g.TX, g.TY);
@@ -147,12 +143,7 @@ extern "C" int mhd_step_noalloc(const mhd_config* cfg, void* cuda_stream, const 
     a.Uout = Uout;
     e = launch_stage(prec, 2, g.TX, g.TY, nblocks, smem, st, g, a);
   }
-  for (int v = 0; v < 5 && e == cudaSuccess; ++v)
-    e = cudaMemcpyAsync(cell_out[v], (char*)Uout + (size_t)v * g.ncell * elem, (size_t)g.ncell * elem,
-                        cudaMemcpyDeviceToDevice, st);
-  for (int d = 0; d < 3 && e == cudaSuccess; ++d)
-    e = cudaMemcpyAsync(face_out[d], (char*)Uout + (size_t)g.face_off[d] * elem,
-                        (size_t)internal_face_count(g, d) * elem, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess) e = copy_state_on_device(g, false, (char*)Uout, elem, cell_out, face_out, st);
   // status word and the CFL max used by the step, read into host stack memory
   unsigned long long hw[4] = {0, 0, 0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(hw, words, sizeof hw, cudaMemcpyDeviceToHost, st);

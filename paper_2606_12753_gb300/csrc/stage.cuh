@@ -176,6 +176,43 @@ __host__ __device__ inline int wrapc(int i, int n, int bc) {
   return i < 0 ? 0 : (i >= n ? n - 1 : i);
 }
 
+// Cells of a pass over all cells: a warp takes runs of up to `run` cells of one (j, k)
+// row, lanes along x, so that the index arithmetic (two divisions) is one per
+// run.  A cell's faces are stored ones: the face above the last cell of a
+// periodic axis is face 0, an outflow axis stores it.
+
+struct RowRun {
+  long long cell, x, ylo, yhi, zlo, zhi;   // index of the row's cell 0 and of its faces in the packed state
+  int i0, i1;
+};
+__device__ __forceinline__ RowRun row_run(const Geo& g, long long item, int per_row, int run) {
+  const long long row = item / per_row;
+  const int j = (int)(row % g.n[1]), k = (int)(row / g.n[1]);
+  const int jh = j + 1 < g.nf[1] ? j + 1 : 0, kh = k + 1 < g.nf[2] ? k + 1 : 0;
+  const long long nx = g.n[0];
+  RowRun r;
+  r.cell = nx * row;
+  r.x = g.face_off[0] + g.nf[0] * row;
+  r.ylo = g.face_off[1] + nx * (j + (long long)g.nf[1] * k);
+  r.yhi = g.face_off[1] + nx * (jh + (long long)g.nf[1] * k);
+  r.zlo = g.face_off[2] + nx * (j + (long long)g.n[1] * k);
+  r.zhi = g.face_off[2] + nx * (j + (long long)g.n[1] * kh);
+  r.i0 = (int)(item - row * per_row) * run;
+  r.i1 = min(r.i0 + run, g.n[0]);
+  return r;
+}
+
+// Run length and grid (8 warps a block) of such a pass: runs of 128 cells where
+// they fill the chip, of 32 in smaller boxes (128 x 128 x 1 FP64: CFL reduction
+// 26 us, 38 with 128-cell runs).
+inline int row_run_length(const Geo& g) {
+  return (long long)g.n[1] * g.n[2] * ((g.n[0] + 127) / 128) >= 152LL * 64 ? 128 : 32;
+}
+inline unsigned row_run_blocks(const Geo& g, int run) {
+  const long long blocks = ((long long)g.n[1] * g.n[2] * ((g.n[0] + run - 1) / run) + 7) / 8;
+  return (unsigned)(blocks < 152LL * 8 ? blocks : 152LL * 8);
+}
+
 // Stored face reference along a normal axis for a (possibly ghost) face
 // index i: value = f(a) + t (f(b) - f(a)).  Periodic axes wrap; outflow axes
 // use the stored faces 0..n and extrapolate linearly beyond them (the ghost
@@ -325,7 +362,7 @@ struct TmaMaps {
 // tm: tensor maps of a.Win for the plain stage kernels, or null (no TMA)
 cudaError_t launch_stage(int prec, int stage, int tx, int ty, unsigned nblocks, size_t smem, cudaStream_t st,
                          const Geo& g, const StageArgs& a, const TmaMaps* tm = nullptr);
-cudaError_t launch_prims(int prec, unsigned nblocks, cudaStream_t st, const Geo& g, const StageArgs& a);
+cudaError_t launch_prims(int prec, cudaStream_t st, const Geo& g, const StageArgs& a);
 cudaError_t stage_set_smem(int prec, int tx, int ty, size_t bytes);
 size_t stage_smem_bytes(int prec, int tx, int ty);
 bool stage_tile_supported(int prec, int tx, int ty);

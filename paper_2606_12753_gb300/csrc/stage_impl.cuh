@@ -1583,72 +1583,79 @@ __global__ void __launch_bounds__(256, PREC == P_FP64 ? 1 : 2) stage_kernel_char
                                                                                                    smem_raw);
 }
 
-// Primitives (and the CFL max) of a state set from outside.  One CTA per
-// (j, k) row of cells, threads along x: the row's index math is one division
-// per CTA, and a cell's faces are its own (the face above the last cell of a
-// periodic axis is face 0), so no ghost logic is needed.  Floor hits count
+// Primitives (and the CFL max) of a state set from outside.  Warps take runs
+// of up to `run` cells of one (j, k) row (row_run), lanes along x; warp of
+// nwarps says which.  A cell's faces are its own (the face above the last cell
+// of a periodic axis is face 0), so no ghost logic is needed.  Floor hits count
 // like those of the stage kernels' recoveries.
 template <int PREC>
-__global__ void __launch_bounds__(128) prims_kernel(Geo g, StageArgs a) {
+__device__ __forceinline__ void prims_rows(const Geo& g, const StageArgs& a, long long warp, long long nwarps, int run) {
   using R = typename Prec<PREC>::R;
   using S = typename Prec<PREC>::S;
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const long long row = blockIdx.x;             // j + ny k
-  const int j = (int)(row % ny), k = (int)(row / ny);
-  const int jh = j + 1 < g.nf[1] ? j + 1 : 0, kh = k + 1 < g.nf[2] ? k + 1 : 0;
+  const int lane = threadIdx.x & 31;
   const S* U = (const S*)a.U;
   R* Wout = (R*)a.Wout;
-  const long long ybase_lo = g.face_off[1] + (long long)nx * (j + (long long)g.nf[1] * k);
-  const long long ybase_hi = g.face_off[1] + (long long)nx * (jh + (long long)g.nf[1] * k);
-  const long long zbase_lo = g.face_off[2] + (long long)nx * (j + (long long)ny * k);
-  const long long zbase_hi = g.face_off[2] + (long long)nx * (j + (long long)ny * kh);
-  const long long xbase = g.face_off[0] + (long long)g.nf[0] * row;
-  R smax = R(0);
+  const int per_row = (g.n[0] + run - 1) / run;
+  const long long items = (long long)g.n[1] * g.n[2] * per_row;
   bool bad = false;
   unsigned nrho = 0, np = 0;
-  // FP64: the largest CFL speed that other rows have folded in so far
-  const double top = __longlong_as_double((long long)*(volatile unsigned long long*)a.nextword);
-  (void)top;
-  (void)nz;
-  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-    const long long s = i + (long long)nx * row;
-    const int ih = i + 1 < g.nf[0] ? i + 1 : 0;
-    R w[NW];
-    int hr, hp;
+  R smax = R(0);
+  for (long long item = warp; item < items; item += nwarps) {
+    const RowRun r = row_run(g, item, per_row, run);
+    // FP64: the largest CFL speed that other warps have folded in so far
+    double top = 0.0;
+    if constexpr (PREC == P_FP64) top = __longlong_as_double((long long)*(volatile unsigned long long*)a.nextword);
+    for (int i = r.i0 + lane; i < r.i1; i += 32) {
+      const long long s = r.cell + i;
+      const int ih = i + 1 < g.nf[0] ? i + 1 : 0;
+      R w[NW];
+      int hr, hp;
 #ifdef MHD_BOUNDS_CHECK
-    {
-      const long long idx[10] = {4 * g.ncell + s, xbase + i, xbase + ih, ybase_lo + i, ybase_hi + i,
-                                 zbase_lo + i, zbase_hi + i, s, g.face_off[1] - 1, g.total - 1};
-      for (int q = 0; q < 7; ++q) (void)bounds_checked(idx[q], g.total, a.status);
-    }
+      {
+        const long long idx[7] = {4 * g.ncell + s, r.x + i, r.x + ih, r.ylo + i, r.yhi + i, r.zlo + i, r.zhi + i};
+        for (int q = 0; q < 7; ++q) (void)bounds_checked(idx[q], g.total, a.status);
+      }
 #endif
-    recover<PREC>(g, (double)U[s], (double)U[g.ncell + s], (double)U[2 * g.ncell + s], (double)U[3 * g.ncell + s],
-                  (double)U[4 * g.ncell + s], (double)U[xbase + i], (double)U[xbase + ih], (double)U[ybase_lo + i],
-                  (double)U[ybase_hi + i], (double)U[zbase_lo + i], (double)U[zbase_hi + i], w, hr, hp);
-    nrho += hr;
-    np += hp;
-    if (not_finite_sums(w)) bad = true;
+      recover<PREC>(g, (double)U[s], (double)U[g.ncell + s], (double)U[2 * g.ncell + s], (double)U[3 * g.ncell + s],
+                    (double)U[4 * g.ncell + s], (double)U[r.x + i], (double)U[r.x + ih], (double)U[r.ylo + i],
+                    (double)U[r.yhi + i], (double)U[r.zlo + i], (double)U[r.zhi + i], w, hr, hp);
+      nrho += hr;
+      np += hp;
+      if (not_finite_sums(w)) bad = true;
 #pragma unroll
-    for (int v = 0; v < NW; ++v) Wout[MHD_IDX(v * g.ncell + s, NW * g.ncell, a.status)] = w[v];
-    if constexpr (PREC == P_FP64) {
-      if (top > 0.0 && !cfl_may_exceed(g, w, top)) continue;
+      for (int v = 0; v < NW; ++v) Wout[MHD_IDX(v * g.ncell + s, NW * g.ncell, a.status)] = w[v];
+      if constexpr (PREC == P_FP64) {
+        if (top > 0.0 && !cfl_may_exceed(g, w, top)) continue;
+      }
+      const R sp = cfl_speed<R>(g, w);
+      smax = sp > smax ? sp : smax;
     }
-    const R sp = cfl_speed<R>(g, w);
-    smax = sp > smax ? sp : smax;
+    if constexpr (PREC == P_FP64) {   // at once, so that the warps after this one form fewer sums
+      double m = smax;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = rmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0 && m > top) atomicMax(a.nextword, (unsigned long long)__double_as_longlong(m));
+    }
   }
   const unsigned mask = 0xffffffffu;
   const unsigned anybad = __any_sync(mask, bad);
   nrho = __reduce_add_sync(mask, nrho);
   np = __reduce_add_sync(mask, np);
-  double sm64 = (double)smax;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sm64 = fmax(sm64, __shfl_xor_sync(mask, sm64, o));
-  if ((threadIdx.x & 31) == 0) {
+  for (int o = 16; o > 0; o >>= 1) smax = rmax(smax, __shfl_xor_sync(mask, smax, o));
+  if (lane == 0) {
     if (anybad) atomicOr(a.status, (unsigned)ST_NONFINITE);
     if (nrho) atomicAdd(&a.counters[C_RHO_FLOOR], (unsigned long long)nrho);
     if (np) atomicAdd(&a.counters[C_P_FLOOR], (unsigned long long)np);
-    if (sm64 > 0.0) atomicMax(a.nextword, (unsigned long long)__double_as_longlong(sm64));
+    if (PREC != P_FP64 && smax > R(0))
+      atomicMax(a.nextword, (unsigned long long)__double_as_longlong((double)smax));
   }
+}
+
+template <int PREC>
+__global__ void __launch_bounds__(256) prims_kernel(Geo g, StageArgs a, int run) {
+  const int warps = blockDim.x / 32;
+  prims_rows<PREC>(g, a, blockIdx.x * (long long)warps + threadIdx.x / 32, gridDim.x * (long long)warps, run);
 }
 
 }  // namespace mhd

@@ -61,9 +61,9 @@ size_t MHD_UNIT_FN(smem_bytes_learned)() {
                                                                   Prec<MHD_UNIT_PREC>::S, false, true>();
 }
 
-cudaError_t MHD_UNIT_FN(launch_prims)(unsigned nblocks, cudaStream_t st, const Geo& g, const StageArgs& args) {
-  (void)nblocks;   // one CTA per (j, k) row of cells
-  prims_kernel<MHD_UNIT_PREC><<<(unsigned)((long long)g.n[1] * g.n[2]), 128, 0, st>>>(g, args);
+cudaError_t MHD_UNIT_FN(launch_prims)(cudaStream_t st, const Geo& g, const StageArgs& args) {
+  const int run = row_run_length(g);
+  prims_kernel<MHD_UNIT_PREC><<<row_run_blocks(g, run), 256, 0, st>>>(g, args, run);
   return cudaGetLastError();
 }
 

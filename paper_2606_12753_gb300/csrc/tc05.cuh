@@ -14,6 +14,13 @@
 // over K = 32 is two instructions with the start addresses advanced by
 // 2 * LBO = 256 bytes.
 //
+// The same bytes read the other way round -- rows as the K dimension, columns
+// as M or N -- are the canonical MN-major layout: a core matrix is then 8 rows
+// (K) of 8 contiguous M or N elements, the stride between groups of 8 columns
+// is the descriptor's stride offset (SBO) and the stride between groups of 8
+// rows its leading offset (LBO).  A product over the rows of two such operands
+// (a weight gradient) needs no transposed copies.
+//
 // The accumulator D (M = 128 rows x N columns, FP32) occupies TMEM lanes
 // 0..127 (row r in lane r) and N consecutive columns; warp w of the CTA may
 // read lanes 32w..32w+31, i.e. its own 32 rows.
@@ -44,6 +51,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 // bits 17-22, M / 16 in bits 24-28.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// The same with both operands MN-major (bits 15 and 16).
+__host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N) {
+  return idesc_bf16_f32(M, N) | (1u << 15) | (1u << 16);
 }
 
 // TMEM allocation of ncols columns (a power of two >= 32) by one whole warp;

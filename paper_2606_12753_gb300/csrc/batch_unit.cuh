@@ -46,7 +46,8 @@ size_t MHD_UNIT_FN(batch_smem_bytes)(int tx, int ty) {
   using S = Prec<MHD_UNIT_PREC>::S;
 #define X(TXv, TYv)                                                                                      \
   if (tx == TXv && ty == TYv)                                                                            \
-    return Tile<TXv, TYv, ring_xo<MHD_UNIT_PREC, FM_PLAIN, BOX_ANY>()>::bytes<                             \
+    return Tile<TXv, TYv, ring_xo<MHD_UNIT_PREC, FM_PLAIN, BOX_ANY>(), false,                            \
+                merge_slopes<MHD_UNIT_PREC, FM_PLAIN, BOX_ANY, TXv, TYv>()>::bytes<                      \
         R, S, slopes_in_smem<MHD_UNIT_PREC, FM_PLAIN, TXv, TYv>(),                                       \
         compact_items<MHD_UNIT_PREC, FM_PLAIN, BOX_ANY, TXv, TYv>()>();
   MHD_BATCH_TILES(X)

@@ -36,11 +36,13 @@ namespace mhd {
 // FLAT: the layout of a two-dimensional box's kernel, which holds one plane
 // of everything and no z-fluxes of the hydro variables (29 KB instead of 75
 // for a 16 x 8 tile of 4-byte primitives).
-template <int TX, int TY, int XO = 2, bool FLAT = false>
+// MERGE: room for the slopes of a plane ahead (kMerge below).
+template <int TX, int TY, int XO = 2, bool FLAT = false, bool MERGE = false>
 struct Tile {
   static constexpr int XOFF = XO;
   static constexpr int nPlanes = FLAT ? 1 : 4;   // ring slots
   static constexpr int nPar = FLAT ? 1 : 2;      // copies of what is kept by plane parity
+  static constexpr int nBn = MERGE ? 4 : nPar;   // planes of lower-face fields
   static constexpr int W = TX + 2 * XO, H = TY + 4;
   static constexpr int nR = W * H;
   // lower-face normal fields of a plane: rows -1..TY of the ring (the rows
@@ -55,7 +57,7 @@ struct Tile {
   // offsets in units of R
   static constexpr int oP = 0;
   static constexpr int oBN = oP + nPlanes * 8 * nR;
-  static constexpr int oHX = oBN + nPar * nBslot;
+  static constexpr int oHX = oBN + nBn * nBslot;
   static constexpr int oHY = oHX + 5 * nX;
   static constexpr int oHZ = oHY + 5 * nY;
   static constexpr int oXC = oHZ + (FLAT ? 0 : 5 * nZ);
@@ -78,9 +80,11 @@ struct Tile {
   static_assert((W + H) % 2 == 0, "the CFL word needs 8-byte alignment");
   // then four mbarriers (8 bytes each), one per ring slot, for TMA planes
   // per-cell half slopes (type R) over the (TX+2) x (TY+2) cells the faces touch:
-  // x and y slopes of the current plane, z slopes of two planes (by parity)
+  // x and y slopes of the current plane, z slopes of two planes (by parity);
+  // MERGE: x and y slopes of two planes, z slopes of three; a flat tile has no
+  // z slopes
   static constexpr int nSl = 7 * nZ;
-  static constexpr int nSlope = (FLAT ? 2 : 4) * nSl;   // (a flat tile has no z slopes)
+  static constexpr int nSlope = (FLAT ? 2 : MERGE ? 7 : 4) * nSl;
   // byte offsets of the regions after the R arrays: the learned switch's
   // queue (QUEUE only), the int tables, the mbarriers
   template <typename R, bool QUEUE>
@@ -185,6 +189,19 @@ constexpr bool slopes_in_smem() {
 // and 632 / 679).
 enum BoxKind { BOX_ANY = 0, BOX_3D = 1, BOX_2D = 2 };
 
+// Whether a kernel forms the slopes of the plane after next inside the flux
+// phase, from the same tickets, instead of in a phase of its own before it:
+// the FP64 kernels with a slope phase, where it fits one CTA's shared memory
+// (217 KB for 16 x 8; 8 x 8 tiles run two CTAs per SM).  The slope phase kept
+// the FP64 pipe half idle (17 warp items of 21 operations, a barrier, and the
+// update phase beside it); merged, the warps without a cell go from loading a
+// plane straight to flux items.  Measured (128^3, stage 1 / 2): 4891 / 5013 us
+// with the phase, 4798 / 4900 merged.
+template <int PREC, int MODE, int KIND, int TX, int TY>
+__host__ __device__ constexpr bool merge_slopes() {
+  return PREC == P_FP64 && KIND != BOX_2D && TX * TY > 64 && slopes_in_smem<PREC, MODE, TX, TY>();
+}
+
 // Whether a kernel takes interior planes by TMA: the plain single-box stage
 // kernels with 4-byte primitives (mixed, FP32).  The batch kernel gathers
 // every plane: its small outflow boxes have few interior tiles, and a tensor
@@ -229,7 +246,9 @@ struct StageKernel {
   using S = typename Prec<PREC>::S;
   using K = typename Prec<PREC>::K;
   static constexpr bool FLAT = KIND == BOX_2D;
-  using T = Tile<TX, TY, ring_xo<PREC, MODE, KIND>(), FLAT>;
+  static constexpr bool kMerge = merge_slopes<PREC, MODE, KIND, TX, TY>();
+  static_assert(!kMerge || (!SPLIT && MODE != FM_LEARNED), "merged slopes need the dynamic flux phase");
+  using T = Tile<TX, TY, ring_xo<PREC, MODE, KIND>(), FLAT, kMerge>;
   static constexpr int W = T::W;
   static constexpr int XO = T::XOFF;
   // TMA planes: plain kernels with 4-byte primitives
@@ -242,7 +261,14 @@ struct StageKernel {
                           (T::nBslot * sizeof(R)) % 128 == 0 && (T::W * sizeof(R)) % 16 == 0),
                 "TMA ring slots must start on 128-byte boundaries and rows span whole 16-byte units");
   // lower-face arrays of plane q, and the index in them of ring cell r
-  static __device__ __forceinline__ const R* bn_slot(const R* sm, int q) { return sm + T::oBN + (q & 1) * T::nBslot; }
+  static __device__ __forceinline__ const R* bn_slot(const R* sm, int q) {
+    return sm + T::oBN + (q & (T::nBn - 1)) * T::nBslot;
+  }
+  // half slopes of plane q along each axis
+  static __device__ __forceinline__ R* slope_slot(R* sl, int axis, int q) {
+    if (kMerge) return sl + (axis < 2 ? 2 * axis + (q & 1) : 4 + (q + 3) % 3) * T::nSl;
+    return sl + (axis < 2 ? axis : 2 + (q & 1)) * T::nSl;
+  }
   static __device__ __forceinline__ int bn_of(int r) { return r - W; }
 
   // ---------------------------------------------------------------- phase A
@@ -252,7 +278,7 @@ struct StageKernel {
                                                     const int* rowc, double dt, int gi0, int gj0, int m,
                                                     bool write_bn, int t0 = 0) {
     R* P = sm + T::oP + (m & 3) * 8 * T::nR;
-    R* BN = sm + T::oBN + (m & 1) * T::nBslot;
+    R* BN = sm + T::oBN + (m & (T::nBn - 1)) * T::nBslot;
     const bool zin = g.bc[2] == 0 || (m >= 0 && m < g.n[2]);
     const int ck = wrapc(m, g.n[2], g.bc[2]);
     const R* Win = (const R*)a.Win;
@@ -508,76 +534,110 @@ struct StageKernel {
 #pragma unroll
         for (int v = 0; v < 7; ++v) out[v] = mc_half_slope(c[0][v], c[1][v], c[2][v]);
       }
-      R* dst = D == 0 ? sl : (D == 1 ? sl + T::nSl : sl + (2 + (q & 1)) * T::nSl);
+      R* dst = slope_slot(sl, D, q);
 #pragma unroll
       for (int v = 0; v < 7; ++v) dst[v * n + cidx] = out[v];
     }
   }
 
-  // Phase B with the slopes of phase B0: per face item, the two cells across
-  // the face, their slopes, PLM values, Riemann flux.
-  static __device__ __forceinline__ void fluxes_sl(const Geo& g, R* sm, const R* sl, int k, int q, bool with_z) {
+  // One flux item with the slopes of phase B0: the two cells across the face,
+  // their slopes, PLM values, Riemann flux, store.
+  static __device__ __forceinline__ void flux_item_sl(const Geo& g, R* sm, R* sl, int k, int q, int nZ, int w, R gam,
+                                                      R ig) {
+    const R* Pq = sm + T::oP + (q & 3) * 8 * T::nR;
+    const R* BNq = bn_slot(sm, q);
+    constexpr int n = T::nZ;
+    R c1[7], c2[7], s1[7], s2[7], wl[7], wr[7], f[7], bn, cm;
+    int o, D, ia, ib;   // ia, ib: slope indices of the two cells
+    const R* sa;
+    const R* sb;
+    if (w < nZ) {
+      const int i = w % (TX + 2) - 1, j = w / (TX + 2) - 1;
+      const int r = MHD_SIDX((i + XO) + W * (j + 2), T::nR);
+      gather<2>(sm + T::oP + (k & 3) * 8 * T::nR, T::nR, r, c1);
+      gather<2>(sm + T::oP + ((k + 1) & 3) * 8 * T::nR, T::nR, r, c2);
+      bn = bn_slot(sm, k + 1)[2 * T::nB + MHD_SIDX(bn_of(r), T::nB)];
+      ia = ib = w;
+      sa = slope_slot(sl, 2, k);
+      sb = slope_slot(sl, 2, k + 1);
+      o = w;
+      D = 2;
+    } else if (w < nZ + T::nX) {
+      o = w - nZ;
+      const int i = o % (TX + 1), j = o / (TX + 1) - 1;
+      const int r = MHD_SIDX(MHD_SIDX((i + XO) + W * (j + 2) - 1, T::nR - 1) + 1, T::nR);
+      gather<0>(Pq, T::nR, r - 1, c1);
+      gather<0>(Pq, T::nR, r, c2);
+      bn = BNq[MHD_SIDX(bn_of(r), T::nB)];
+      ia = i + (TX + 2) * (j + 1);
+      ib = ia + 1;
+      sa = sb = slope_slot(sl, 0, q);
+      D = 0;
+    } else {
+      o = w - nZ - T::nX;
+      const int i = o % (TX + 2) - 1, j = o / (TX + 2);
+      const int r = MHD_SIDX(MHD_SIDX((i + XO) + W * (j + 2) - W, T::nR - W) + W, T::nR);
+      gather<1>(Pq, T::nR, r - W, c1);
+      gather<1>(Pq, T::nR, r, c2);
+      bn = BNq[T::nB + MHD_SIDX(bn_of(r), T::nB)];
+      ib = (i + 1) + (TX + 2) * (j + 1);
+      ia = ib - (TX + 2);
+      sa = sb = slope_slot(sl, 1, q);
+      D = 1;
+    }
+#pragma unroll
+    for (int v = 0; v < 7; ++v) {
+      s1[v] = sa[v * n + ia];
+      s2[v] = sb[v * n + ib];
+      wl[v] = c1[v] + s1[v];
+      wr[v] = c2[v] - s2[v];
+    }
+    wl[0] = rmax(wl[0], gpar<R>(g.rho_floor, g.frho_floor));
+    wr[0] = rmax(wr[0], gpar<R>(g.rho_floor, g.frho_floor));
+    wl[4] = rmax(wl[4], gpar<R>(g.p_floor, g.fp_floor));
+    wr[4] = rmax(wr[4], gpar<R>(g.p_floor, g.fp_floor));
+    solve(g, wl, wr, bn, gam, ig, f, &cm);
+    store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
+  }
+
+  // Phase B with the slopes of phase B0
+  static __device__ __forceinline__ void fluxes_sl(const Geo& g, R* sm, R* sl, int k, int q, bool with_z) {
     const int nZ = with_z ? T::nZ : 0;
     const int nitems = nZ + T::nX + T::nY;
     const R gam = gpar<R>(g.gamma, g.fgamma);
     const R ig = R(1) / (gam - R(1));
-    const R* Pq = sm + T::oP + (q & 3) * 8 * T::nR;
-    const R* BNq = bn_slot(sm, q);
-    constexpr int n = T::nZ;
-    for (int w = threadIdx.x; w < nitems; w += blockDim.x) {
-      R c1[7], c2[7], s1[7], s2[7], wl[7], wr[7], f[7], bn, cm;
-      int o, D, ia, ib;   // ia, ib: slope indices of the two cells
-      const R* sa;
-      const R* sb;
-      if (w < nZ) {
-        const int i = w % (TX + 2) - 1, j = w / (TX + 2) - 1;
-        const int r = MHD_SIDX((i + XO) + W * (j + 2), T::nR);
-        gather<2>(sm + T::oP + (k & 3) * 8 * T::nR, T::nR, r, c1);
-        gather<2>(sm + T::oP + ((k + 1) & 3) * 8 * T::nR, T::nR, r, c2);
-        bn = bn_slot(sm, k + 1)[2 * T::nB + MHD_SIDX(bn_of(r), T::nB)];
-        ia = ib = w;
-        sa = sl + (2 + (k & 1)) * T::nSl;
-        sb = sl + (2 + ((k + 1) & 1)) * T::nSl;
-        o = w;
-        D = 2;
-      } else if (w < nZ + T::nX) {
-        o = w - nZ;
-        const int i = o % (TX + 1), j = o / (TX + 1) - 1;
-        const int r = MHD_SIDX(MHD_SIDX((i + XO) + W * (j + 2) - 1, T::nR - 1) + 1, T::nR);
-        gather<0>(Pq, T::nR, r - 1, c1);
-        gather<0>(Pq, T::nR, r, c2);
-        bn = BNq[MHD_SIDX(bn_of(r), T::nB)];
-        ia = i + (TX + 2) * (j + 1);
-        ib = ia + 1;
-        sa = sb = sl;
-        D = 0;
-      } else {
-        o = w - nZ - T::nX;
-        const int i = o % (TX + 2) - 1, j = o / (TX + 2);
-        const int r = MHD_SIDX(MHD_SIDX((i + XO) + W * (j + 2) - W, T::nR - W) + W, T::nR);
-        gather<1>(Pq, T::nR, r - W, c1);
-        gather<1>(Pq, T::nR, r, c2);
-        bn = BNq[T::nB + MHD_SIDX(bn_of(r), T::nB)];
-        ib = (i + 1) + (TX + 2) * (j + 1);
-        ia = ib - (TX + 2);
-        sa = sb = sl + T::nSl;
-        D = 1;
-      }
-#pragma unroll
-      for (int v = 0; v < 7; ++v) {
-        s1[v] = sa[v * n + ia];
-        s2[v] = sb[v * n + ib];
-        wl[v] = c1[v] + s1[v];
-        wr[v] = c2[v] - s2[v];
-      }
-      wl[0] = rmax(wl[0], gpar<R>(g.rho_floor, g.frho_floor));
-      wr[0] = rmax(wr[0], gpar<R>(g.rho_floor, g.frho_floor));
-      wl[4] = rmax(wl[4], gpar<R>(g.p_floor, g.fp_floor));
-      wr[4] = rmax(wr[4], gpar<R>(g.p_floor, g.fp_floor));
-      solve(g, wl, wr, bn, gam, ig, f, &cm);
-      store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
-    }
+    for (int w = threadIdx.x; w < nitems; w += blockDim.x) flux_item_sl(g, sm, sl, k, q, nZ, w, gam, ig);
     cell_emf(sm, q, threadIdx.x, blockDim.x);
+  }
+
+  // Phase B with the slopes of plane k + 2 formed beside the fluxes (kMerge):
+  // warps draw the flux items, then the slope items, from one ticket counter.
+  // The slopes read plane k + 3, which the threads without a cell have just
+  // loaded; a warp waits for it on mbarrier `ready` (one arrival of each of
+  // those threads a plane) before its first slope item, so no warp waits for
+  // another's flux items.
+  static __device__ __forceinline__ void fluxes_merged(const Geo& g, const StageArgs& a, R* sm, R* sl, int k,
+                                                       bool with_z, bool with_slopes, int* ticket,
+                                                       unsigned long long* ready, unsigned& phases) {
+    const int nZ = with_z ? T::nZ : 0;
+    const int nitems = nZ + T::nX + T::nY;
+    const int nfaces = (nitems + 31) / 32 * 32, nslopes = with_slopes ? 3 * T::nZ : 0;
+    const R gam = gpar<R>(g.gamma, g.fgamma);
+    const R ig = R(1) / (gam - R(1));
+    if ((int)threadIdx.x >= T::nC) cell_emf(sm, k + 1, (int)threadIdx.x - T::nC, (int)blockDim.x - T::nC);
+    const int lane = threadIdx.x & 31;
+    const auto draw = [&] {
+      int t = 0;
+      if (lane == 0) t = atomicAdd(ticket, 32);
+      return __shfl_sync(0xffffffffu, t, 0);
+    };
+    int t = draw();
+    for (; t < nfaces; t = draw())
+      if (t + lane < nitems) flux_item_sl(g, sm, sl, k, k + 1, nZ, t + lane, gam, ig);
+    if (!with_slopes) return;
+    tma_wait(a, ready, 0, phases);
+    for (; t < nfaces + nslopes; t = draw())
+      if (t - nfaces + lane < nslopes) slope_item(g, sm, sl, k + 2, t - nfaces + lane);
   }
 
   // The z-faces of a two-dimensional box: both states are the cell's own
@@ -1463,6 +1523,14 @@ struct StageKernel {
       fluxes_learned(g, a, sm, queue, qcnt, kb - 2, kb - 1, false, gi0, gj0, kb, ke, nh, nd);
       __syncthreads();
     }
+    if constexpr (kMerge) {
+      if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"((int)blockDim.x - T::nC)
+                     : "memory");
+      }
+      slopes(g, sm, sl, kb - 1, false, nullptr);
+      __syncthreads();
+    }
     ZCarry zc{S(0), R(0), false};   // face group: upper z-face of the previous plane
     for (int k = LEARN ? kb - 1 : kb - 2; k < ke; ++k) {
       // the threads without a cell in the update phase load the next plane
@@ -1470,7 +1538,13 @@ struct StageKernel {
       const bool first = !LEARN && k == kb - 2;   // its planes are in
       const bool tma_next = !first && plane_tma(k + 2);
       const int nl = (int)blockDim.x - T::nC;   // threads without a cell in the update phase
-      if (first) {
+      if constexpr (kMerge) {
+        // plane k + 3, for the slopes of plane k + 2
+        if (k + 3 <= ke + 1 && (int)threadIdx.x >= T::nC) {
+          load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 3, true, T::nC);
+          asm volatile("{\n .reg .b64 s;\n mbarrier.arrive.shared::cta.b64 s, [%0];\n}" ::"r"(smem_u32(mbar)) : "memory");
+        }
+      } else if (first) {
       } else if (kDyn && !tma_next && nl >= 32 && nl % 32 == 0) {
         if ((int)threadIdx.x >= T::nC) {
           load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 2, true, T::nC);
@@ -1484,7 +1558,9 @@ struct StageKernel {
         if (!(kDyn && tma_next)) __syncthreads();
       }
       if (tma_next) tma_wait(a, mbar, (k + 2) & 3, phases);
-      if constexpr (SLOPES) {
+      if constexpr (kMerge) {
+        fluxes_merged(g, a, sm, sl, k, !first, k + 3 <= ke + 1, ticket + (k & 1), mbar, phases);
+      } else if constexpr (SLOPES) {
         slopes(g, sm, sl, k + 1, false, ticket + (k & 1));
         __syncthreads();
         fluxes_sl(g, sm, sl, k, k + 1, !first);
@@ -1514,6 +1590,9 @@ struct StageKernel {
       if (k >= kb) update_plane(g, a, sm, sdt, gi0, gj0, k, nrho, np, bad, smax, zc, top, kPF ? &pre : nullptr);
     }
 
+    if constexpr (kMerge) {   // every wait on it precedes the last barrier
+      if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(mbar)) : "memory");
+    }
     finish(a, nrho, np, nh, nd, bad, smax);
     if (ntma && threadIdx.x == 0) atomicAdd(&a.counters[C_TMA], (unsigned long long)ntma);
     fold_bounds_flag(a);

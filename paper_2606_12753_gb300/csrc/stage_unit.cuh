@@ -42,7 +42,8 @@ size_t MHD_UNIT_FN(smem_bytes)(int tx, int ty) {
   using S = Prec<MHD_UNIT_PREC>::S;
 #define X(TXv, TYv)                                                                                      \
   if (tx == TXv && ty == TYv)                                                                            \
-    return Tile<TXv, TYv, ring_xo<MHD_UNIT_PREC, FM_PLAIN, BOX_3D>()>::bytes<                              \
+    return Tile<TXv, TYv, ring_xo<MHD_UNIT_PREC, FM_PLAIN, BOX_3D>(), false,                             \
+                merge_slopes<MHD_UNIT_PREC, FM_PLAIN, BOX_3D, TXv, TYv>()>::bytes<                       \
         R, S, slopes_in_smem<MHD_UNIT_PREC, FM_PLAIN, TXv, TYv>()>();
   MHD_TILES(X)
 #undef X
@@ -51,8 +52,9 @@ size_t MHD_UNIT_FN(smem_bytes)(int tx, int ty) {
 
 // characteristic reconstruction (16 x 8 tile) keeps its slopes in shared memory
 size_t MHD_UNIT_FN(smem_bytes_char)() {
-  return Tile<16, 8, ring_xo<MHD_UNIT_PREC, FM_CHAR, BOX_ANY>()>::bytes<Prec<MHD_UNIT_PREC>::R, Prec<MHD_UNIT_PREC>::S,
-                                                               true>();
+  return Tile<16, 8, ring_xo<MHD_UNIT_PREC, FM_CHAR, BOX_ANY>(), false,
+              merge_slopes<MHD_UNIT_PREC, FM_CHAR, BOX_ANY, 16, 8>()>::bytes<Prec<MHD_UNIT_PREC>::R,
+                                                                             Prec<MHD_UNIT_PREC>::S, true>();
 }
 
 // the learned switch (16 x 8 tile) queues its face items in shared memory

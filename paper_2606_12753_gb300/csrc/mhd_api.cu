@@ -1114,7 +1114,7 @@ __device__ __forceinline__ float cfl_bound(const Geo& g, float rho, const float 
 __device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double (&m)[3], double e,
                                           const double (&b)[3]) {
   if (lt_(rho, g.rho_floor)) rho = g.rho_floor;
-  const double ir = rcp_(rho);
+  const double ir = qrcp_(rho);
   const double b2[3] = {b[0] * b[0], b[1] * b[1], b[2] * b[2]};
   const double bb = b2[0] + b2[1] + b2[2];
   double p = g.gm1 * (e - 0.5 * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) * ir - 0.5 * bb);
@@ -1124,8 +1124,8 @@ __device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (g.n[d] > 1) {
-      const double root = root_(xx + a4r * (b2[(d + 1) % 3] + b2[(d + 2) % 3]));
-      sum += (fabs(m[d]) * ir + root_(0.5 * (s + root))) * g.inv_d[d];
+      const double root = qroot_(xx + a4r * (b2[(d + 1) % 3] + b2[(d + 2) % 3]));
+      sum += (fabs(m[d]) * ir + qroot_(0.5 * (s + root))) * g.inv_d[d];
     }
   }
   return sum;

@@ -108,16 +108,60 @@ __host__ __device__ __forceinline__ double rsqrt_(double x) {   // square root
   return sqrt(x);
 #endif
 }
-// The same root one operation shorter: the refinement applied to x y0
-// (used where the result may round differently).
-__host__ __device__ __forceinline__ double root_(double x) {
+// The same three with fewer FP64-pipe operations again (rcp 2, rsqrt and root
+// 3), where the result may round differently (the characteristic slopes and
+// the lean solvers below).  With the residual e of the seed y the result is
+// y (1 + e + e^2) (rcp), y (1 + e/2 + 3/8 e^2) (the roots); the last term,
+// ~1e-12 of y, is formed in FP32 and added to y's bits as an integer number of
+// ulps, and the step to the result is one fma.  Halving is an exponent
+// decrement.  A face has nine of them: 128^3 HLLD 4787 / 4900 -> 4573 / 4676 us.
+// (Adding e^2 to e's own bits instead is exact to fewer ulps but needs a test
+// for the next binade, which cost more than the operations it saved.)
+#ifdef __CUDA_ARCH__
+// y (1 + (EIGHTHS / 8) e^2), y normal, |e| < 1e-4 (half an ulp from rounding; a
+// step into the next binade, one in 10^12, is off by at most the step)
+template <int EIGHTHS>
+__device__ __forceinline__ double plus_square(double y, double e) {
+  const unsigned he = (unsigned)__double2hiint(e) & 0x7fffffffu;
+  // |e| and y's mantissa in [1, 2), cut to FP32 (|e| to 0 below 2^-62: its square is below an ulp)
+  const float ef = he < 0x3c100000u ? 0.0f : __uint_as_float((he << 3) - (896u << 23));
+  const float my = __uint_as_float(((unsigned)__double2hiint(y) << 3 & 0x007fffffu) | 0x3f800000u);
+  const int ulps = __float2int_rn(ef * ef * (my * (0.125f * EIGHTHS * 4503599627370496.0f)));
+  return __longlong_as_double(__double_as_longlong(y) + ulps);
+}
+__device__ __forceinline__ double half_(double x) {   // normal x
+  return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x));
+}
+#endif
+__host__ __device__ __forceinline__ double qrcp_(double x) {
+#ifdef __CUDA_ARCH__
+  if (!f64_plain(x)) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, e, plus_square<8>(r, e));
+#else
+  return 1.0 / x;
+#endif
+}
+__host__ __device__ __forceinline__ double qrsqrt_(double x) {
+#ifdef __CUDA_ARCH__
+  if (!f64_plain(x) || __double2hiint(x) < 0) return 1.0 / sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(half_(y), e, plus_square<3>(y, e));
+#else
+  return 1.0 / sqrt(x);
+#endif
+}
+__host__ __device__ __forceinline__ double qroot_(double x) {
 #ifdef __CUDA_ARCH__
   if (!f64_plain(x) || __double2hiint(x) < 0) return sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double t = x * y;
-  const double h = fma(-t, y, 1.0);
-  return fma(t, h * fma(0.375, h, 0.5), t);
+  const double t = x * y, e = fma(-t, y, 1.0);
+  return fma(half_(t), e, plus_square<3>(t, e));
 #else
   return sqrt(x);
 #endif
@@ -125,7 +169,9 @@ __host__ __device__ __forceinline__ double root_(double x) {
 __host__ __device__ __forceinline__ float rcp_(float x) { return 1.0f / x; }
 __host__ __device__ __forceinline__ float rrsqrt_(float x) { return rsqrtf(x); }
 __host__ __device__ __forceinline__ float rsqrt_(float x) { return sqrtf(x); }
-__host__ __device__ __forceinline__ float root_(float x) { return sqrtf(x); }
+__host__ __device__ __forceinline__ float qrcp_(float x) { return 1.0f / x; }
+__host__ __device__ __forceinline__ float qrsqrt_(float x) { return rsqrtf(x); }
+__host__ __device__ __forceinline__ float qroot_(float x) { return sqrtf(x); }
 
 // Sign-bit helpers (integer operations: they keep the sign tests of the
 // limiter off the FP64 pipe).
@@ -143,6 +189,15 @@ __host__ __device__ __forceinline__ bool opposite_signs(float a, float b) {
   return (a < 0.0f) != (b < 0.0f) && a != 0.0f && b != 0.0f;
 #endif
 }
+// x with its sign flipped where f is set (on the integer pipe in FP64)
+__host__ __device__ __forceinline__ double flip_(double x, bool f) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(x) ^ (f ? (int)0x80000000 : 0), __double2loint(x));
+#else
+  return f ? -x : x;
+#endif
+}
+
 __host__ __device__ __forceinline__ double copysign_(double m, double s) { return copysign(m, s); }
 __host__ __device__ __forceinline__ float copysign_(float m, float s) { return copysignf(m, s); }
 __host__ __device__ __forceinline__ double fmin_(double a, double b) {
@@ -408,26 +463,17 @@ __host__ __device__ __forceinline__ void hlld_flux(const R* wl, const R* wr, R b
 // Measured (GB300, 128^3, stage 1 / 2 in us): HLLD 7197 / 7678 with the plain
 // solvers, 5521 / 5984 with these; HLL 5487 / 5967 and 5031 / 5515.
 
-// x with its sign flipped where f is set (on the integer pipe in FP64)
-__host__ __device__ __forceinline__ double flip_(double x, bool f) {
-#ifdef __CUDA_ARCH__
-  return __hiloint2double(__double2hiint(x) ^ (f ? (int)0x80000000 : 0), __double2loint(x));
-#else
-  return f ? -x : x;
-#endif
-}
-
 // The larger fast speed of two states, b2_* = |B|^2 and bt2_* = |B_t|^2 of each.
 __host__ __device__ __forceinline__ double max_fast_speed(const double* wl, const double* wr, double b2_l, double b2_r,
                                                           double bt2_l, double bt2_r, double gamma) {
   const double g4 = 4.0 * gamma;
   const double x_l = gamma * wl[4] - b2_l, x_r = gamma * wr[4] - b2_r;
-  const double t_l = gamma * wl[4] + b2_l + root_(x_l * x_l + (g4 * wl[4]) * bt2_l);
-  const double t_r = gamma * wr[4] + b2_r + root_(x_r * x_r + (g4 * wr[4]) * bt2_r);
+  const double t_l = gamma * wl[4] + b2_l + qroot_(x_l * x_l + (g4 * wl[4]) * bt2_l);
+  const double t_r = gamma * wr[4] + b2_r + qroot_(x_r * x_r + (g4 * wr[4]) * bt2_r);
   const bool l = lt_(t_r * wl[0], t_l * wr[0]);
   const double t = l ? t_l : t_r, rho = l ? wl[0] : wr[0];
   // sqrt(t / (2 rho)) = t / sqrt(2 rho t)
-  return t * (0.70710678118654752440 * rrsqrt_(rho * t));
+  return t * (0.70710678118654752440 * qrsqrt_(rho * t));
 }
 
 // Whether a star state's denominator den = num - bn^2 counts as zero:
@@ -453,14 +499,14 @@ __host__ __device__ __forceinline__ LeanStar lean_star(double v, double w, doubl
   LeanStar st;
   const double num = m * ssm, den = num - bn2;
   st.degen = star_degenerate(den, num, bn2);
-  const double t = smu * rcp_(den);
+  const double t = smu * qrcp_(den);
   const double c1 = st.degen ? 0.0 : bn * t;          // v* = v - B_t c1
   const double c2 = st.degen ? 1.0 : 1.0 + m * t;    // B_t* = B_t c2, c2 = (m (S - u) - bn^2) / den
   st.v = v - by * c1;
   st.w = w - bz * c1;
   st.by = by * c2;
   st.bz = bz * c2;
-  st.y = rrsqrt_(num);
+  st.y = qrsqrt_(num);
   st.sq = rabs(m) * st.y;
   st.isq = rabs(ssm) * st.y;
   return st;
@@ -509,7 +555,7 @@ __host__ __device__ __forceinline__ void hlld_flux_lean(const double* wl, const 
   // the outer sides' S - u, m = rho (S - u) and the contact speed S_M
   const double sdl = sl - wl[1], sdr = sr - wr[1];
   const double ml = wl[0] * sdl, mr = wr[0] * sdr;
-  const double sm = ((ptl - ptr) + mr * wr[1] - ml * wl[1]) * rcp_(mr - ml);
+  const double sm = ((ptl - ptr) + mr * wr[1] - ml * wl[1]) * qrcp_(mr - ml);
   const bool left = outside ? out_l : ge0(sm);
   // A: the side that holds the face, B: the other one
   const double rho = left ? wl[0] : wr[0], u = left ? wl[1] : wr[1], p = left ? wl[4] : wr[4];
@@ -547,7 +593,7 @@ __host__ __device__ __forceinline__ void hlld_flux_lean(const double* wl, const 
                                       left ? wr[6] : wl[6], bn, bn2, left ? mr : ml, sb - sm,
                                       sm - (left ? wr[1] : wl[1]));
       const bool neg = lt0(bn) == left;   // sign of sgn(bn) (+ on the left, - on the right)
-      const double is = rcp_(A.sq + B.sq);
+      const double is = qrcp_(A.sq + B.sq);
       const double ps = flip_(A.sq * B.sq, neg);
       fby = (A.sq * B.by + B.sq * A.by + ps * (B.v - A.v)) * is;
       fbz = (A.sq * B.bz + B.sq * A.bz + ps * (B.w - A.w)) * is;
@@ -575,7 +621,7 @@ __host__ __device__ __forceinline__ void hll_flux_lean(const double* wl, const d
   const double cm = max_fast_speed(wl, wr, b2l, b2r, bt2l, bt2r, gamma);
   *cmax = cm;
   const double sl = rmin(wl[1], wr[1]) - cm, sr = rmax(wl[1], wr[1]) + cm;
-  const double is = rcp_(sr - sl);
+  const double is = qrcp_(sr - sl);
   double a = sr * is, b = -(sl * is), c = sl * a;
   if (ge0(sl)) { a = 1.0; b = c = 0.0; }   // outside the fan: one side's flux
   else if (le0(sr)) { b = 1.0; a = c = 0.0; }
@@ -668,7 +714,7 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
                                                     R* slope) {
   const R rho = w0[0];
   const R ir = rcp_(rho);
-  const R a2 = gamma * w0[4] * ir, a = root_(a2), sr = root_(rho), isr = rcp_(sr);
+  const R a2 = gamma * w0[4] * ir, a = rsqrt_(a2), sr = rsqrt_(rho), isr = rcp_(sr);
   const R bnr = bn0 * isr, b1 = w0[5] * isr, b2 = w0[6] * isr;
   const R bt2 = b1 * b1 + b2 * b2, bsq = bnr * bnr + bt2;
   // forms without cancellation: c_f^2 - c_s^2 = sqrt((a^2-b^2)^2 + 4 a^2 b_t^2),
@@ -681,9 +727,9 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
   const R sq = sqrt((a2 - bsq) * (a2 - bsq) + R(4) * a2 * bt2);
   const R cf2 = R(0.5) * (a2 + bsq + sq);
   const R cs2 = gt0(cf2) ? a2 * bnr * bnr * rcp_(cf2) : R(0);
-  const R cf = root_(cf2), cs = root_(cs2), bt = root_(bt2);
+  const R cf = rsqrt_(cf2), cs = rsqrt_(cs2), bt = rsqrt_(bt2);
   R be1, be2;
-  if (lt_(Eps<R>::degen * root_(a2 + bsq), bt)) {
+  if (lt_(Eps<R>::degen * rsqrt_(a2 + bsq), bt)) {
     const R ib = rcp_(bt);
     be1 = b1 * ib;
     be2 = b2 * ib;
@@ -694,8 +740,8 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
   if (lt_(Eps<R>::degen * cf2, sq)) {
     const R id = rcp_(sq);
     const R fa = R(0.5) * (bsq - a2 + sq), as2 = R(0.5) * (a2 - bsq + sq);   // c_f^2 - a^2, a^2 - c_s^2
-    af = root_((gt0(as2) ? as2 : R(0)) * id);
-    as = root_((gt0(fa) ? fa : R(0)) * id);
+    af = rsqrt_((gt0(as2) ? as2 : R(0)) * id);
+    as = rsqrt_((gt0(fa) ? fa : R(0)) * id);
   } else {
     af = R(1);
     as = R(0);
@@ -740,6 +786,89 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
   const R tb = a * sr * (as * Fp - af * Sp);
   slope[5] = be1 * tb - sr * be2 * Ap;
   slope[6] = be2 * tb + sr * be1 * Ap;
+}
+
+// The same in FP64, with a third fewer operations: reciprocals and roots from
+// one reciprocal root each, the projection's coefficients formed once for both
+// sides, and of c_f^2 - a^2 and a^2 - c_s^2 the smaller one from their product
+// a^2 b_t^2 (exactly zero when B_t is), so that the root of the discriminant
+// needs no correct rounding.  Measured (96x64x80, stage 1 / 2): 2138 / 2125 ->
+// 1854 / 1842 us with the shorter roots; against 80-bit arithmetic its error is
+// 0.75 of the plain one's on random states and a hundredth of it where B_t is
+// small.
+__host__ __device__ __forceinline__ void char_half_slope(const double* wm, const double* w0, const double* wp, double bn0,
+                                                         double gamma, double* slope) {
+  const double rho = w0[0], gp = gamma * w0[4];
+  const double isr = qrsqrt_(rho), sr = rho * isr, ir = isr * isr;
+  const double a2 = gp * ir, ra = qrsqrt_(a2), a = a2 * ra, ia2 = ra * ra;
+  const double bnr = bn0 * isr, b1 = w0[5] * isr, b2 = w0[6] * isr;
+  const double bt2 = b1 * b1 + b2 * b2, bsq = bnr * bnr + bt2;
+  const double d = a2 - bsq, s = a2 + bsq, q = 4.0 * a2 * bt2, disc = d * d + q;
+  double be1, be2;
+  if (lt_(Eps<double>::degen * Eps<double>::degen * s, bt2)) {
+    const double ib = qrsqrt_(bt2);
+    be1 = b1 * ib;
+    be2 = b2 * ib;
+  } else {
+    be1 = be2 = 0.70710678118654752440;
+  }
+  const double iq = gt0(disc) ? qrsqrt_(disc) : 0.0, sq = disc * iq;   // c_f^2 - c_s^2 and its reciprocal
+  const double cf2 = 0.5 * (s + sq), icf = qrsqrt_(cf2);
+  const double cf = cf2 * icf, cs = a * (rabs(bnr) * icf);
+  double af, as;
+  if (lt_(Eps<double>::degen * cf2, sq)) {
+    const double big = 0.5 * (rabs(d) + sq), small = quarter_(q) * qrcp_(big);
+    const bool pos = ge0(d);   // a^2 - c_s^2 is the larger one
+    af = qroot_((pos ? big : small) * iq);
+    as = qroot_((pos ? small : big) * iq);
+  } else {
+    af = 1.0;
+    as = 0.0;
+  }
+  const bool neg = lt0(bn0);   // sgn(bn) = -1
+  const double fc = af * cf, sc = as * cs, h = 0.5 * ia2, hs = 0.5 * isr, hr = h * ir, ha = hs * ra;
+  const double x1 = fc * h, x2 = sc * h, y1 = af * hr, y2 = as * hr, z1 = af * ha, z2 = as * ha;
+  const double e1 = flip_(0.5 * be1, neg), e2 = flip_(0.5 * be2, neg), g1 = be1 * hs, g2 = be2 * hs;
+  const double x1s = flip_(x1, neg), x2s = flip_(x2, neg);
+  double dc[7];   // limited wave amplitudes: f-, a-, s-, e, s+, a+, f+
+  {
+    double m[7], p[7];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const double* lo = side == 0 ? wm : w0;
+      const double* hi = side == 0 ? w0 : wp;
+      double v[7];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) v[k] = hi[k] - lo[k];
+      const double t = be1 * v[2] + be2 * v[3], bb = be1 * v[5] + be2 * v[6];
+      const double xf = x1 * v[1] - x2s * t, yf = y1 * v[4] + z2 * bb;
+      const double xs = x2 * v[1] + x1s * t, ys = y2 * v[4] - z1 * bb;
+      const double xa = e2 * v[2] - e1 * v[3], ya = g1 * v[6] - g2 * v[5];
+      double* c = side == 0 ? m : p;
+      c[0] = yf - xf;
+      c[1] = ya - xa;
+      c[2] = ys - xs;
+      c[3] = v[0] - v[4] * ia2;
+      c[4] = ys + xs;
+      c[5] = ya + xa;
+      c[6] = yf + xf;
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k) dc[k] = mc_lim_half(m[k], p[k]);
+  }
+  const double Fp = dc[6] + dc[0], Fm = dc[6] - dc[0];
+  const double Sp = dc[4] + dc[2], Sm = dc[4] - dc[2];
+  const double Ap = sr * (dc[5] + dc[1]), Am = dc[5] - dc[1];
+  const double w = af * Fp + as * Sp;
+  slope[0] = rho * w + dc[3];
+  slope[1] = fc * Fm + sc * Sm;
+  const double tv = fc * Sm - sc * Fm;
+  slope[2] = flip_(be1 * tv + be2 * Am, neg);
+  slope[3] = flip_(be2 * tv - be1 * Am, neg);
+  slope[4] = gp * w;
+  const double tb = (a * sr) * (as * Fp - af * Sp);
+  slope[5] = be1 * tb - be2 * Ap;
+  slope[6] = be2 * tb + be1 * Ap;
 }
 
 // Characteristic PLM of a face: as plm_face, with the slopes of c1 and c2

@@ -5,7 +5,12 @@
 // the larger of max(|rho (S-u)(S-S_M)|, bn^2) / |den| of its two sides: the
 // star states divide by den, whose own rounding error that ratio amplifies;
 // both solvers take tens of roundings.  A side that both solvers count as
-// degenerate (|den| well inside the threshold) divides by nothing.
+// degenerate (|den| well inside the threshold) divides by nothing.  Also the
+// reciprocals and roots those solvers use, against IEEE: within 2^-50 (a few
+// roundings) over exponents 2^-300..2^300, and the IEEE value of zeros,
+// subnormals, infinities, NaN and (roots) negative numbers; and the FP64
+// characteristic half slope against the plain one, within 256 eps of the
+// differences it limits, where the plain one does not cancel.
 #include <cstdio>
 #include <cstring>
 #include <cuda_runtime.h>
@@ -94,26 +99,73 @@ __host__ __device__ double face_excess(int kind, unsigned long long q, bool hll)
   return worst / (64.0 * eps * kappa + dc);
 }
 
-__global__ void check(int kind, bool hll, unsigned long long n, unsigned long long* word) {
+__host__ __device__ inline double relative(double got, double ref) {
+  if (got != got || ref != ref) return got != got && ref != ref ? 0.0 : 1.0;
+  if (got == ref) return 0.0;
+  return ref == 0.0 || ref - ref != 0.0 ? 1.0 : fabs(got - ref) / fabs(ref);
+}
+__host__ __device__ double math_excess(int kind, unsigned long long q, bool) {
+  const double special[10] = {0.0, -0.0, 4.9e-324, -4.9e-324, 1.0 / 0.0, -1.0 / 0.0, 0.0 / 0.0, 2.2e-308, -1.0, -2.5};
+  const unsigned long long z = mix64(q), e = 723 + (z >> 52) % 601;
+  union { unsigned long long u; double d; } bits;
+  bits.u = (e << 52) | (mix64(z) & 0xfffffffffffffull);
+  const double x = q < 10 ? special[q] : kind == 0 && (z & 1) ? -bits.d : bits.d;
+  const double got = kind == 0 ? qrcp_(x) : kind == 1 ? qrsqrt_(x) : qroot_(x);
+  const double ref = kind == 0 ? 1.0 / x : kind == 1 ? 1.0 / sqrt(x) : sqrt(x);
+  return relative(got, ref) / (q < 10 ? 1e-300 : 8.881784197001252e-16);   // 2^-50
+}
+__host__ __device__ double slope_excess(int kind, unsigned long long q, bool) {
+  Rng g{mix64(q * 8 + kind + 77)};
+  const double jump = kind == 0 ? 0.5 : 1e-2;
+  double base[7], w[3][7], a[7], b[7], bn = g.u(-2, 2);
+  for (int i = 0; i < 7; ++i) base[i] = i == 0 ? exp(g.u(-2, 2)) : i == 4 ? exp(g.u(-3, 2)) : g.u(-1, 1);
+  if (kind == 2) bn = 0.0;
+  if (kind == 3) base[5] = base[6] = 0.0;
+  for (int s = 0; s < 3; ++s)
+    for (int i = 0; i < 7; ++i)
+      w[s][i] = i == 0 || i == 4 ? base[i] * exp(0.5 * jump * g.u(-1, 1)) : base[i] + jump * g.u(-1, 1);
+  if (kind == 3) w[1][5] = w[1][6] = 0.0;
+  char_half_slope<double>(w[0], w[1], w[2], bn, 5.0 / 3.0, a);
+  char_half_slope(w[0], w[1], w[2], bn, 5.0 / 3.0, b);
+  // the plain one takes the root of a difference of a^2, b^2 and their
+  // discriminant's root: its rounding error relative to what is left is
+  // amplified by a^2 over a^2 b_t^2 / (a^2 + b^2)
+  const double ir = 1.0 / w[1][0], a2 = 5.0 / 3.0 * w[1][4] * ir;
+  const double bt2 = (w[1][5] * w[1][5] + w[1][6] * w[1][6]) * ir, s = a2 + bn * bn * ir + bt2;
+  const double kappa = kind == 3 ? 1.0 : 1.0 + s * s / (a2 * bt2 < 1e-3 * s * s ? 0.0 : a2 * bt2);
+  double worst = 0.0, norm = 0.0;
+  for (int i = 0; i < 7; ++i) {
+    const double m = fabs(w[1][i] - w[0][i]) + fabs(w[2][i] - w[1][i]);
+    norm += m * m;
+  }
+  for (int i = 0; i < 7; ++i) worst = fmax(worst, fabs(a[i] - b[i]));
+  return worst / (sqrt(norm) * (256.0 * 2.220446049250313e-16) * kappa);
+}
+
+enum { FLUX, MATH, SLOPE };
+__host__ __device__ inline double excess(int what, int kind, unsigned long long q, bool hll) {
+  return what == FLUX ? face_excess(kind, q, hll) : what == MATH ? math_excess(kind, q, hll) : slope_excess(kind, q, hll);
+}
+__global__ void check(int what, int kind, bool hll, unsigned long long n, unsigned long long* word) {
   double m = 0.0;
   for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < n;
        q += (unsigned long long)gridDim.x * blockDim.x)
-    m = fmax(m, face_excess(kind, q, hll));
+    m = fmax(m, excess(what, kind, q, hll));
   atomicMax(word, (unsigned long long)__double_as_longlong(m));
 }
 
-double worst(bool host, int kind, bool hll) {
+double worst(bool host, int what, int kind, bool hll) {
   double m = 0.0;
   if (host) {
     for (unsigned long long q = 0; q < 200000; ++q) {
-      const double e = face_excess(kind, q, hll);
+      const double e = excess(what, kind, q, hll);
       m = e > m ? e : m;
     }
     return m;
   }
   unsigned long long* d;
   if (cudaMalloc(&d, 8) != cudaSuccess || cudaMemset(d, 0, 8) != cudaSuccess) return 1e30;
-  check<<<512, 128>>>(kind, hll, 1ull << 22, d);
+  check<<<512, 128>>>(what, kind, hll, 1ull << 22, d);
   if (cudaMemcpy(&m, d, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return 1e30;
   return m;
 }
@@ -123,7 +175,10 @@ int main(int argc, char** argv) {
   printf("{");
   for (int hll = 0; hll < 2; ++hll)
     for (int kind = 0; kind < 5; ++kind)
-      printf("%s\"%s%d\": %.3g", hll + kind ? ", " : "", hll ? "hll" : "hlld", kind, worst(host, kind, hll));
+      printf("%s\"%s%d\": %.3g", hll + kind ? ", " : "", hll ? "hll" : "hlld", kind, worst(host, FLUX, kind, hll));
+  const char* names[3] = {"rcp", "rsqrt", "root"};
+  for (int kind = 0; kind < 3; ++kind) printf(", \"%s\": %.3g", names[kind], worst(host, MATH, kind, false));
+  for (int kind = 0; kind < 4; ++kind) printf(", \"slope%d\": %.3g", kind, worst(host, SLOPE, kind, false));
   printf("}\n");
   return 0;
 }

@@ -3,7 +3,8 @@ fluxes with fewer operations, against the plain ones (tests/cuda/flux_check.cu,
 built here with nvcc) on random faces: large and small jumps, supersonic
 faces, vanishing fields, equal states and degenerate star states.  The
 difference stays within 64 roundings times the conditioning of the star
-states."""
+states.  The reciprocals, roots and characteristic slopes of the same kernels
+likewise."""
 import json
 import os
 import shutil

@@ -228,6 +228,19 @@ __host__ __device__ constexpr int ring_xo() {
   return tma_planes<PREC, MODE, KIND>() ? 4 : 2;
 }
 
+// Threads per CTA and CTAs per SM of the plain stage kernel: FP64 tiles run
+// 256 threads (1 CTA per SM, 2 for 8x8); the FP32-bulk forms keep 24 warps
+// per SM at about 85 registers a thread: 3 CTAs of 256 threads for tiles of up
+// to 128 columns, 2 of 384 for 192 columns, 1 of 768 for 256 columns.
+template <int PREC, int TX, int TY>
+__host__ __device__ constexpr int stage_threads() {
+  return PREC == P_FP64 ? 256 : (TX * TY >= 256 ? 768 : (TX * TY >= 192 ? 384 : 256));
+}
+template <int PREC, int TX, int TY>
+__host__ __device__ constexpr int stage_min_blocks() {
+  return PREC == P_FP64 ? (TX * TY <= 64 ? 2 : 1) : 768 / stage_threads<PREC, TX, TY>();
+}
+
 // SPLIT: the update phase splits each cell between two threads (face group
 // and conserved group, named-barrier hand-over); the CTA then needs at least
 // two threads per cell of a plane.  The learned-switch kernels of the mixed
@@ -246,6 +259,21 @@ struct StageKernel {
   using S = typename Prec<PREC>::S;
   using K = typename Prec<PREC>::K;
   static constexpr bool FLAT = KIND == BOX_2D;
+  // Threads per CTA, known to the compiler where they may be: the work loops of a plane then have
+  // constant trip counts and their item arithmetic folds, which kernels bound by the instructions
+  // that they issue and fetch feel.  Stages 1/2 in us, before -> after, all bit for bit alike:
+  // mixed 256^3 2582/2802 -> 2383/2584, FP32 256^3 2192/2292 -> 2104/2205, FP32 2D 1024^2
+  // 158/173 -> 144/163, mixed characteristic -2.5%, FP64 -0.3%.
+  // Batch and learned kernels of the FP32 bulk read blockDim.x: with the constant the compiler
+  // contracts the same sources in another way (a batch moves by 4e-8, a learned state by 3e-6 in a
+  // few steps) for no gain in time.  The learned flux loops alone keep their bits and take it
+  // (mixed 128^3 1025/1012 -> 1004/990).
+  static constexpr int NT = KIND != BOX_ANY ? stage_threads<PREC, TX, TY>() : 256;
+  static constexpr bool kFixed = KIND != BOX_ANY || MODE == FM_CHAR || (MODE == FM_PLAIN && PREC == P_FP64);
+  static __device__ __forceinline__ int threads() { return kFixed ? NT : (int)blockDim.x; }
+  static __device__ __forceinline__ int flux_threads() {
+    return kFixed || MODE == FM_LEARNED ? NT : (int)blockDim.x;
+  }
   static constexpr bool kMerge = merge_slopes<PREC, MODE, KIND, TX, TY>();
   static_assert(!kMerge || (!SPLIT && MODE != FM_LEARNED), "merged slopes need the dynamic flux phase");
   using T = Tile<TX, TY, ring_xo<PREC, MODE, KIND>(), FLAT, kMerge>;
@@ -272,8 +300,8 @@ struct StageKernel {
   static __device__ __forceinline__ int bn_of(int r) { return r - W; }
 
   // ---------------------------------------------------------------- phase A
-  // Threads [t0, blockDim.x) load, item r = threadIdx.x - t0 with stride
-  // blockDim.x - t0 (t0 > 0 leaves the threads of the update phase out).
+  // Threads [t0, threads()) load, item r = threadIdx.x - t0 with stride
+  // threads() - t0 (t0 > 0 leaves the threads of the update phase out).
   static __device__ __forceinline__ void load_plane(const Geo& g, const StageArgs& a, R* sm, const int* colc,
                                                     const int* rowc, double dt, int gi0, int gj0, int m,
                                                     bool write_bn, int t0 = 0) {
@@ -287,7 +315,7 @@ struct StageKernel {
     // the ring columns the stencil reads: XO - 2 .. XO + TX + 1 (a padded
     // ring's outer columns are for the 16-byte rule of TMA boxes only)
     constexpr int WR = TX + 4;
-    for (int rr = t; rr < WR * T::H; rr += (int)blockDim.x - t0) {
+    for (int rr = t; rr < WR * T::H; rr += threads() - t0) {
       const int x = XO - 2 + rr % WR, y = rr / WR;
       const int r = x + W * y;
       const int gi = gi0 - XO + x, gj = gj0 - 2 + y;
@@ -422,8 +450,8 @@ struct StageKernel {
     const R gam = gpar<R>(g.gamma, g.fgamma);
     const R ig = R(1) / (gam - R(1));
     if (kDyn && ticket) {
-      const int first = (int)blockDim.x > T::nC ? T::nC : 0;   // threads without a cell first
-      if ((int)threadIdx.x >= first) cell_emf(sm, q, (int)threadIdx.x - first, (int)blockDim.x - first);
+      const int first = flux_threads() > T::nC ? T::nC : 0;   // threads without a cell first
+      if ((int)threadIdx.x >= first) cell_emf(sm, q, (int)threadIdx.x - first, flux_threads() - first);
       const int lane = threadIdx.x & 31;
       // kCompact: the tile's list (a chunk's first pass, without z-faces, takes every item)
       const bool listed = kCompact && with_z;
@@ -440,8 +468,8 @@ struct StageKernel {
           flux_item(g, sm, k, q, nZ, listed ? list[MHD_SIDX(base + lane, T::nItems)] : base + lane, gam, ig);
       }
     } else {
-      for (int w = threadIdx.x; w < nitems; w += blockDim.x) flux_item(g, sm, k, q, nZ, w, gam, ig);
-      cell_emf(sm, q, threadIdx.x, blockDim.x);
+      for (int w = threadIdx.x; w < nitems; w += flux_threads()) flux_item(g, sm, k, q, nZ, w, gam, ig);
+      cell_emf(sm, q, threadIdx.x, flux_threads());
     }
   }
 
@@ -500,7 +528,7 @@ struct StageKernel {
         if (first + base + lane < 3 * n) slope_item(g, sm, sl, q, first + base + lane);
       }
     } else {
-      for (int it = first + threadIdx.x; it < 3 * n; it += blockDim.x) slope_item(g, sm, sl, q, it);
+      for (int it = first + threadIdx.x; it < 3 * n; it += flux_threads()) slope_item(g, sm, sl, q, it);
     }
   }
 
@@ -606,8 +634,8 @@ struct StageKernel {
     const int nitems = nZ + T::nX + T::nY;
     const R gam = gpar<R>(g.gamma, g.fgamma);
     const R ig = R(1) / (gam - R(1));
-    for (int w = threadIdx.x; w < nitems; w += blockDim.x) flux_item_sl(g, sm, sl, k, q, nZ, w, gam, ig);
-    cell_emf(sm, q, threadIdx.x, blockDim.x);
+    for (int w = threadIdx.x; w < nitems; w += flux_threads()) flux_item_sl(g, sm, sl, k, q, nZ, w, gam, ig);
+    cell_emf(sm, q, threadIdx.x, flux_threads());
   }
 
   // Phase B with the slopes of plane k + 2 formed beside the fluxes (kMerge):
@@ -624,7 +652,7 @@ struct StageKernel {
     const int nfaces = (nitems + 31) / 32 * 32, nslopes = with_slopes ? 3 * T::nZ : 0;
     const R gam = gpar<R>(g.gamma, g.fgamma);
     const R ig = R(1) / (gam - R(1));
-    if ((int)threadIdx.x >= T::nC) cell_emf(sm, k + 1, (int)threadIdx.x - T::nC, (int)blockDim.x - T::nC);
+    if ((int)threadIdx.x >= T::nC) cell_emf(sm, k + 1, (int)threadIdx.x - T::nC, flux_threads() - T::nC);
     const int lane = threadIdx.x & 31;
     const auto draw = [&] {
       int t = 0;
@@ -654,7 +682,7 @@ struct StageKernel {
     const R gam = gpar<R>(g.gamma, g.fgamma);
     const R ig = R(1) / (gam - R(1));
     R* C = sm + T::oZC;
-    for (int w = (int)blockDim.x - 1 - (int)threadIdx.x; w < T::nZ; w += blockDim.x) {
+    for (int w = flux_threads() - 1 - (int)threadIdx.x; w < T::nZ; w += flux_threads()) {
       const int i = w % (TX + 2) - 1, j = w / (TX + 2) - 1;
       const int r = MHD_SIDX((i + XO) + W * (j + 2), T::nR);
       R c[7], f[7], cm;
@@ -795,7 +823,7 @@ struct StageKernel {
     const R ig = R(1) / (gam - R(1));
     int* cnt = qcnt + 2 * (q & 1);   // [0] HLL items (front), [1] HLLD items (back)
     const bool record = a.choices != nullptr && q >= kb && q < ke;
-    for (int base = threadIdx.x & ~31; base < nitems; base += blockDim.x) {
+    for (int base = threadIdx.x & ~31; base < nitems; base += flux_threads()) {
       const int w = base + lane;
       const bool valid = w < nitems;
       int o = 0, D = 0;
@@ -839,7 +867,7 @@ struct StageKernel {
     __syncthreads();
     const int nhll = cnt[0];
     if (threadIdx.x < 2) qcnt[2 * ((q + 1) & 1) + threadIdx.x] = 0;   // next plane's counters; read before a barrier
-    for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
+    for (int t = threadIdx.x; t < nitems; t += flux_threads()) {
       const int w = queue[t];
       R c[4][7], wl[7], wr[7], f[7], bn, cm;
       int o;
@@ -854,7 +882,7 @@ struct StageKernel {
       }
       store_any(D, g, sm, q, o, f, cm, wl[0], wr[0]);
     }
-    cell_emf(sm, q, threadIdx.x, blockDim.x);
+    cell_emf(sm, q, threadIdx.x, flux_threads());
   }
 
   // ---------------------------------------------------------------- phase C
@@ -870,9 +898,9 @@ struct StageKernel {
     // warps after them, when at least two warps are left for the cells:
     // otherwise the first warps would form both and the last ones idle.
     constexpr int kEdgeThreads = (T::nE + 31) / 32 * 32;
-    const bool apart = (int)blockDim.x >= kEdgeThreads + 64;
+    const bool apart = threads() >= kEdgeThreads + 64;
     const int c0 = apart ? (int)threadIdx.x - kEdgeThreads : (int)threadIdx.x;
-    const int cstep = apart ? (int)blockDim.x - kEdgeThreads : (int)blockDim.x;
+    const int cstep = apart ? threads() - kEdgeThreads : threads();
     for (int c = c0 < 0 ? T::nC : c0; c < T::nC; c += cstep) {
       const int i = c % TX, j = c / TX;
       const int iz = (i + 1) + (TX + 2) * (j + 1);
@@ -898,7 +926,7 @@ struct StageKernel {
     R* EX1 = sm + T::oEXY + sk1 * 2 * T::nE;   // edges at k+1/2
     R* EY1 = EX1 + T::nE;
     constexpr int nX = T::nX, nY = T::nY, nZ = T::nZ;
-    for (int e = threadIdx.x; e < T::nE; e += apart ? kEdgeThreads : (int)blockDim.x) {
+    for (int e = threadIdx.x; e < T::nE; e += apart ? kEdgeThreads : threads()) {
       const int i = e % (TX + 1), j = e / (TX + 1);
       {  // E_z at (i-1/2, j-1/2), plane k
         const int xa = i + (TX + 1) * j, xb = xa + (TX + 1);
@@ -936,9 +964,9 @@ struct StageKernel {
     const R* HY = sm + T::oHY;
     // edge slots on whole warps from warp 0, cells on the warps after them (as in phase C)
     constexpr int kEdgeThreads = (T::nE + 31) / 32 * 32;
-    const bool apart = (int)blockDim.x >= kEdgeThreads + 64;
+    const bool apart = threads() >= kEdgeThreads + 64;
     const int c0 = apart ? (int)threadIdx.x - kEdgeThreads : (int)threadIdx.x;
-    const int cstep = apart ? (int)blockDim.x - kEdgeThreads : (int)blockDim.x;
+    const int cstep = apart ? threads() - kEdgeThreads : threads();
     for (int c = c0 < 0 ? T::nC : c0; c < T::nC; c += cstep) {
       const int i = c % TX, j = c / TX;
       const int ixm = i + (TX + 1) * (j + 1), ixp = ixm + 1;
@@ -960,7 +988,7 @@ struct StageKernel {
     R* EX1 = sm + T::oEXY + slot * 2 * T::nE;
     R* EY1 = EX1 + T::nE;
     constexpr int nX = T::nX, nY = T::nY, nZ = T::nZ;
-    for (int e = threadIdx.x; e < T::nE; e += apart ? kEdgeThreads : (int)blockDim.x) {
+    for (int e = threadIdx.x; e < T::nE; e += apart ? kEdgeThreads : threads()) {
       const int i = e % (TX + 1), j = e / (TX + 1);
       {
         const int xa = i + (TX + 1) * j, xb = xa + (TX + 1);
@@ -1260,7 +1288,7 @@ struct StageKernel {
     const int nx = g.n[0], ny = g.n[1];
     const int t = threadIdx.x;
     if constexpr (kCanSplit) {
-      if (SPLIT || 2 * T::nC <= (int)blockDim.x) {
+      if (SPLIT || 2 * T::nC <= threads()) {
       static_assert(T::nC % 32 == 0, "the split update phase needs whole warps per group");
       double* U5 = reinterpret_cast<double*>(sm + T::oHX);   // [5][nC], in the idle flux arrays
       static_assert((size_t)5 * T::nC * sizeof(double) <= (size_t)T::nHydro * sizeof(R),
@@ -1292,7 +1320,7 @@ struct StageKernel {
       return;
       }
     }
-    for (int c = t; c < T::nC; c += blockDim.x) {
+    for (int c = t; c < T::nC; c += threads()) {
       const int i = c % TX, j = c / TX;
       const int gi = gi0 + i, gj = gj0 + j;
       if (gi >= nx || gj >= ny) continue;
@@ -1396,7 +1424,7 @@ struct StageKernel {
 #ifdef MHD_BOUNDS_CHECK
     if (threadIdx.x == 0) *cta_bounds_flag() = 0u;
 #endif
-    for (int t = threadIdx.x; t < T::W + T::H; t += blockDim.x) {
+    for (int t = threadIdx.x; t < T::W + T::H; t += threads()) {
       if (t < T::W) colc[t] = wrapc(gi0 - XO + t, g.n[0], g.bc[0]);
       else rowc[t - T::W] = wrapc(gj0 - 2 + (t - T::W), g.n[1], g.bc[1]);
     }
@@ -1435,7 +1463,7 @@ struct StageKernel {
       load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, 0, true);
       __syncthreads();
       if constexpr (SLOPES) {
-        for (int it = threadIdx.x; it < 2 * T::nZ; it += blockDim.x) slope_item(g, sm, sl, 0, it);
+        for (int it = threadIdx.x; it < 2 * T::nZ; it += threads()) slope_item(g, sm, sl, 0, it);
         __syncthreads();
         fluxes_sl(g, sm, sl, 0, 0, false);
       } else {
@@ -1461,12 +1489,12 @@ struct StageKernel {
       __syncthreads();
       {
         const R* P0 = sm + T::oP;
-        for (int e = threadIdx.x; e < 8 * T::nR; e += blockDim.x) {
+        for (int e = threadIdx.x; e < 8 * T::nR; e += threads()) {
           const R v = P0[e];
 #pragma unroll
           for (int m = 1; m < 4; ++m) sm[T::oP + m * 8 * T::nR + e] = v;
         }
-        for (int e = threadIdx.x; e < T::nBslot; e += blockDim.x) sm[T::oBN + T::nBslot + e] = sm[T::oBN + e];
+        for (int e = threadIdx.x; e < T::nBslot; e += threads()) sm[T::oBN + T::nBslot + e] = sm[T::oBN + e];
       }
       __syncthreads();
       if constexpr (SLOPES) {
@@ -1525,7 +1553,7 @@ struct StageKernel {
     }
     if constexpr (kMerge) {
       if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"((int)blockDim.x - T::nC)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(threads() - T::nC)
                      : "memory");
       }
       slopes(g, sm, sl, kb - 1, false, nullptr);
@@ -1537,7 +1565,7 @@ struct StageKernel {
       // while the others finish that phase (unless it comes by TMA)
       const bool first = !LEARN && k == kb - 2;   // its planes are in
       const bool tma_next = !first && plane_tma(k + 2);
-      const int nl = (int)blockDim.x - T::nC;   // threads without a cell in the update phase
+      const int nl = threads() - T::nC;   // threads without a cell in the update phase
       if constexpr (kMerge) {
         // plane k + 3, for the slopes of plane k + 2
         if (k + 3 <= ke + 1 && (int)threadIdx.x >= T::nC) {
@@ -1549,12 +1577,12 @@ struct StageKernel {
         if ((int)threadIdx.x >= T::nC) {
           load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 2, true, T::nC);
           asm volatile("bar.sync %0, %1;" ::"r"(kLoadBarrier), "r"(nl) : "memory");
-          asm volatile("bar.arrive %0, %1;" ::"r"(kPlaneBarrier), "r"((int)blockDim.x) : "memory");
+          asm volatile("bar.arrive %0, %1;" ::"r"(kPlaneBarrier), "r"(threads()) : "memory");
         } else {
-          asm volatile("bar.sync %0, %1;" ::"r"(kPlaneBarrier), "r"((int)blockDim.x) : "memory");
+          asm volatile("bar.sync %0, %1;" ::"r"(kPlaneBarrier), "r"(threads()) : "memory");
         }
       } else {
-        if (!tma_next) load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 2, true, T::nC < (int)blockDim.x ? T::nC : 0);
+        if (!tma_next) load_plane(g, a, sm, colc, rowc, dt, gi0, gj0, k + 2, true, T::nC < threads() ? T::nC : 0);
         if (!(kDyn && tma_next)) __syncthreads();
       }
       if (tma_next) tma_wait(a, mbar, (k + 2) & 3, phases);
@@ -1609,19 +1637,6 @@ struct StageKernel {
 #endif
   }
 };
-
-// Threads per CTA and CTAs per SM of the plain stage kernel: FP64 tiles run
-// 256 threads (1 CTA per SM, 2 for 8x8); the FP32-bulk forms keep 24 warps
-// per SM at about 85 registers a thread: 3 CTAs of 256 threads for tiles of up
-// to 128 columns, 2 of 384 for 192 columns, 1 of 768 for 256 columns.
-template <int PREC, int TX, int TY>
-__host__ __device__ constexpr int stage_threads() {
-  return PREC == P_FP64 ? 256 : (TX * TY >= 256 ? 768 : (TX * TY >= 192 ? 384 : 256));
-}
-template <int PREC, int TX, int TY>
-__host__ __device__ constexpr int stage_min_blocks() {
-  return PREC == P_FP64 ? (TX * TY <= 64 ? 2 : 1) : 768 / stage_threads<PREC, TX, TY>();
-}
 
 // CTAs per SM of the kernel of a two-dimensional box: its flat tile leaves the
 // shared memory of a second FP64 CTA.

@@ -274,48 +274,82 @@ extern "C" void mhd_default_config(mhd_config* c, int nx, int ny, int nz) {
 
 // ---- z-chunk length ---------------------------------------------------------
 // The device time of a launch whose CTAs march chunks of planes, in units of
-// a lone CTA's plane: `groups` lists (planes of a chunk, number of chunks) in
-// the order they start; `slots` CTAs are resident on kSMs SMs at once.  A chunk
-// costs its planes and a prologue (three plane loads and 1.65 flux passes, and
-// the loads' latency).  A plane takes slowdown(r) with r CTAs on an SM: an
-// FP64 CTA keeps the FP64 pipe busy by itself, the others hide each other's
-// latencies (measured: 5.4, 6.8 and 8.7 us for a mixed plane with 1, 2, 3).
+// a lone CTA's plane.  `groups` lists (planes of a chunk, number of chunks) in
+// the order they start; each of the kSMs SMs holds up to `most` CTAs and takes
+// the next chunk when one of its own ends.  The CTAs of an SM do not share it
+// evenly: the one that started first issues first and runs ahead, so that a
+// launch of one wave ends with its SMs half empty (mixed 240^3: 240 planes a
+// chunk 2304 us a stage, 32 planes 2042).  rate[n - 1] holds the planes per
+// unit of an SM's n CTAs, oldest first.  A chunk costs its planes and a
+// prologue.  SMs in the same state advance together.
 struct ChunkGroup {
   int planes;
   long long count;
 };
 static constexpr int kSMs = 152;
 
-static double march_time(const std::vector<ChunkGroup>& groups, int slots, bool fp64, double prologue) {
-  struct Running {
-    double left;
-    long long count;
+struct MarchRates {
+  int most;
+  double rate[3][3];
+  double prologue;
+};
+
+// FP64 CTAs share the FP64 pipe, which one of them keeps busy.  The rates of
+// the others are a fit to 260 measured stages (16 sizes of 48^3 to 320^3 at all
+// chunk lengths, mixed and FP32; the estimates are 2.6 % off in the mean, FP64
+// 0.8 %).
+static MarchRates march_rates(bool fp64, int most) {
+  if (fp64) return {most, {{1.0}, {0.5, 0.5}, {1.0 / 3, 1.0 / 3, 1.0 / 3}}, 1.8};
+  return {most, {{1.0}, {0.90, 0.75}, {0.825, 0.67, 0.515}}, 1.65};
+}
+
+static double march_time(std::vector<ChunkGroup> groups, const MarchRates& m) {
+  struct SMs {
+    int count, n;
+    double left[3];   // of the resident chunks, oldest first
   };
-  std::vector<Running> run;
-  long long active = 0;
-  size_t next = 0;
-  long long waiting = groups.empty() ? 0 : groups[0].count;
+  std::vector<SMs> sms{{kSMs, 0, {}}}, merged;
   double time = 0.0;
-  for (int event = 0; event < 4096; ++event) {
-    while (active < slots && next < groups.size()) {
-      const long long n = std::min<long long>(slots - active, waiting);
-      if (n) run.push_back({groups[next].planes + prologue, n});
-      active += n;
-      waiting -= n;
-      if (waiting == 0 && ++next < groups.size()) waiting = groups[next].count;
+  size_t next = 0;
+  for (int event = 0; event < 1 << 14; ++event) {
+    for (int n = 0; n < m.most; ++n)   // waiting chunks go to the emptiest SMs first
+      for (size_t i = 0; i < sms.size(); ++i) {
+        while (next < groups.size() && groups[next].count == 0) ++next;
+        if (next == groups.size()) break;
+        if (sms[i].n != n) continue;
+        const int take = (int)std::min<long long>(sms[i].count, groups[next].count);
+        if (take < sms[i].count) {
+          SMs rest = sms[i];
+          rest.count -= take;
+          sms[i].count = take;
+          sms.push_back(rest);
+        }
+        sms[i].left[sms[i].n++] = groups[next].planes + m.prologue;
+        groups[next].count -= take;
+      }
+    double step = HUGE_VAL;
+    for (const SMs& c : sms)
+      for (int i = 0; i < c.n; ++i) step = std::min(step, c.left[i] / m.rate[c.n - 1][i]);
+    if (step == HUGE_VAL) return time;
+    time += step;
+    merged.clear();
+    for (const SMs& c : sms) {
+      SMs d = {c.count, 0, {}};
+      for (int i = 0; i < c.n; ++i) {
+        const double left = c.left[i] - step * m.rate[c.n - 1][i];
+        if (left > 1e-6) d.left[d.n++] = left;
+      }
+      const auto alike = [&](const SMs& e) {
+        if (e.n != d.n) return false;
+        for (int i = 0; i < d.n; ++i)
+          if (std::fabs(e.left[i] - d.left[i]) > 1e-4) return false;
+        return true;
+      };
+      const auto it = std::find_if(merged.begin(), merged.end(), alike);
+      if (it == merged.end()) merged.push_back(d);
+      else it->count += d.count;
     }
-    if (run.empty()) return time;
-    double step = run[0].left;
-    for (const Running& r : run) step = std::min(step, r.left);
-    const double per_sm = std::max(1.0, (double)active / kSMs);
-    time += step * (fp64 ? per_sm : 0.7 + 0.3 * per_sm);
-    size_t keep = 0;
-    for (Running& r : run) {
-      r.left -= step;
-      if (r.left > 1e-9) run[keep++] = r;
-      else active -= r.count;
-    }
-    run.resize(keep);
+    sms.swap(merged);
   }
   return HUGE_VAL;
 }
@@ -328,32 +362,32 @@ static int resident_ctas(const mhd_config* c, int tx, int ty) {
 }
 
 // Default planes per z-chunk: 32, unless march_time finds a length that takes
-// less than 0.94 of it.  Small boxes then have chunks enough for every SM
-// (24^3 FP64: 1 plane, 125 us a stage, 1048 with one chunk of 24; 64^3 mixed: 5,
-// 72 and 196) and middle ones no nearly empty last wave (128^3 mixed: 43, 437
-// and 483; 96x64x80 FP32: 10, 109 and 179).  The estimate is a few percent off
-// where the choices are close, hence the margin.  Results do not depend on it,
-// but for the learned switch in FP32 arithmetic, whose first pass over a
-// chunk rounds differently: it keeps 32.
+// less than 0.98 of it.  Small boxes then have chunks enough for every SM (us a
+// stage: 24^3 FP64 1 plane a chunk 112, one chunk of 24 989; 64^3 mixed 5: 68,
+// 32: 186) and middle ones no nearly empty last wave (128^3 FP64 16: 4713, 32:
+// 5094; 128^3 mixed 15: 377, 32: 461; 97x130x75 FP32 13: 210, 32: 240; 240^3
+// mixed stays at 32: 2048, one chunk of 240: 2306).  On 17 sizes from 24^3 to
+// 352^3 and all precisions the choice took at most 1.7 % more than the best length.
+// Results do not depend on it, but for the learned switch in FP32 arithmetic,
+// whose first pass over a chunk rounds differently: it keeps 32.
 static int default_chunk(const mhd_config* c, int tx, int ty) {
   if (c->nz <= 1 || (c->riemann == MHD_LEARNED && c->precision != MHD_FP64)) return 32;
   const long long columns = (long long)((c->nx + tx - 1) / tx) * ((c->ny + ty - 1) / ty);
-  const bool fp64 = c->precision == MHD_FP64;
-  const int slots = kSMs * resident_ctas(c, tx, ty);
+  const MarchRates rates = march_rates(c->precision == MHD_FP64, resident_ctas(c, tx, ty));
   const auto estimate = [&](int tz) {
     const int n = (c->nz + tz - 1) / tz, last = c->nz - (n - 1) * tz;
     std::vector<ChunkGroup> groups;
     if (n > 1) groups.push_back({tz, columns * (n - 1)});
     groups.push_back({last, columns});
-    return march_time(groups, slots, fp64, fp64 ? 2.1 : 3.5);
+    return march_time(groups, rates);
   };
   int best = 32;
   const double base = estimate(32);
-  double least = 0.94 * base;
+  double least = 0.98 * base;
   for (int n = 1, tz = c->nz, previous = 0; n <= c->nz; ++n, previous = tz) {
     tz = (c->nz + n - 1) / n;
     if (tz == previous || tz > (1 << 20)) continue;
-    if (tz < 16 && columns * n > 40LL * slots) break;   // shorter chunks only add prologues to a full chip
+    if (tz < 16 && columns * n > 40LL * kSMs * rates.most) break;   // shorter chunks only add prologues to a full chip
     const double t = estimate(tz);
     if (t < least) {
       least = t;
@@ -1371,12 +1405,14 @@ static void drop_graph(mhd_batch* b) {
 }
 
 // Default planes per z-chunk of a batch: the length whose items, started
-// longest first, take the least estimated time, if that is under 0.97 of 32's
-// (measured, FP32, us a stage: 64 boxes of 32-128 cells an axis 4705 at 32,
-// 4574 at 64; 4 boxes of 32-112 360 at 32, 200 at 12).
+// longest first, take the least estimated time, if that is under 0.98 of 32's
+// (measured, FP32, us a stage: 64 boxes of 32-128 cells an axis 4690 at 32,
+// 4598 at 96; 4 boxes of 32-112 365 at 32, 198 at 8).  An item's prologue also
+// draws its ticket and gathers its planes without TMA: 2.5 planes.
 static int batch_default_chunk(const mhd_batch* b, int tx, int ty) {
   static const int lengths[] = {32, 2, 4, 6, 8, 12, 16, 24, 48, 64, 96, 128};
-  const int slots = kSMs * resident_ctas(&b->cfg[0], tx, ty);
+  MarchRates rates = march_rates(b->prec == MHD_FP64, resident_ctas(&b->cfg[0], tx, ty));
+  if (b->prec != MHD_FP64) rates.prologue = 2.5;
   int best = 32;
   double least = HUGE_VAL;
   for (int tz : lengths) {
@@ -1389,11 +1425,11 @@ static int batch_default_chunk(const mhd_batch* b, int tx, int ty) {
       count[c.nz - (n - 1) * tz] += columns;
       items += columns * n;
     }
-    if (tz < 16 && items > 40LL * slots) continue;
+    if (tz < 16 && items > 40LL * kSMs * rates.most) continue;
     std::vector<ChunkGroup> groups;
     for (const auto& q : count) groups.push_back({q.first, q.second});
-    const double t = march_time(groups, slots, b->prec == MHD_FP64, b->prec == MHD_FP64 ? 2.1 : 2.5);
-    if (tz == 32) least = 0.97 * t;
+    const double t = march_time(groups, rates);
+    if (tz == 32) least = 0.98 * t;
     else if (t < least) {
       least = t;
       best = tz;

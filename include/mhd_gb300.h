@@ -272,8 +272,8 @@ int mhd_get_stats(mhd_handle* h, mhd_stats* out);
  * both solvers (Sec. 2.2, HLLD_Solver and HLL_Solver in Tables 2-4); the
  * network is this library's addition.  Inference and training use BF16
  * tensor-core MMAs with FP32 accumulation: mlp_forward and mlp_backward run
- * the 128-row products on the tcgen05 tensor cores (accumulators in tensor
- * memory), the weight gradients (32 output rows) on warp-level MMAs.
+ * every product over the rows, the weight gradients included, on the tcgen05
+ * tensor cores (accumulators in tensor memory).
  *
  * Parameter block: mlp_param_bytes() bytes of device memory, caller-owned:
  * FP32 master parameters in the order W1[32][16], b1[32], W2[32][32], b2[32],
@@ -295,6 +295,9 @@ int mlp_backward(const void* block, const float* features, const float* labels, 
  * (1633 floats each, zero-initialised by the caller); refreshes the bf16 copies. */
 int mlp_adam(void* block, float* m, float* v, const float* grad, int step, double lr, double beta1, double beta2,
              double eps, void* cuda_stream);
+/* One training step: zeroes grad, then mlp_backward and mlp_adam. */
+int mlp_train_step(void* block, const float* features, const float* labels, long long n, float* grad, float* m,
+                   float* v, int step, double lr, double beta1, double beta2, double eps, void* cuda_stream);
 /* Training data from the current state of a periodic box: for each face id
  * (d * nx*ny*nz + cell index, the face below that cell along axis d) the 16
  * features of its reconstructed states and the label 1 when the HLLD and HLL

@@ -265,9 +265,9 @@ struct StageKernel {
   // mixed 256^3 2582/2802 -> 2383/2584, FP32 256^3 2192/2292 -> 2104/2205, FP32 2D 1024^2
   // 158/173 -> 144/163, mixed characteristic -2.5%, FP64 -0.3%.
   // Batch and learned kernels of the FP32 bulk read blockDim.x: with the constant the compiler
-  // contracts the same sources in another way (a batch moves by 4e-8, a learned state by 3e-6 in a
-  // few steps) for no gain in time.  The learned flux loops alone keep their bits and take it
-  // (mixed 128^3 1025/1012 -> 1004/990).
+  // contracts the same sources in another way, and a batch moves by 4e-8, a learned state by 3e-6 in
+  // a few steps.  The learned flux loops alone keep their bits and take it (mixed 128^3 1025/1012 ->
+  // 1004/990).
   static constexpr int NT = KIND != BOX_ANY ? stage_threads<PREC, TX, TY>() : 256;
   static constexpr bool kFixed = KIND != BOX_ANY || MODE == FM_CHAR || (MODE == FM_PLAIN && PREC == P_FP64);
   static __device__ __forceinline__ int threads() { return kFixed ? NT : (int)blockDim.x; }

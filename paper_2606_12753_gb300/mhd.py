@@ -71,7 +71,7 @@ EXPORTS = ["mhd_default_config", "mhd_create", "mhd_set_state", "mhd_get_state",
            "mhd_batch_step_async", "mhd_batch_set_tile", "mhd_batch_get_tile", "mhd_batch_autotune",
            "mhd_batch_set_barrier_timeout", "mhd_batch_inject_missed_arrival", "mhd_batch_box_dt",
            "mhd_batch_get_stats", "mhd_batch_destroy", "mhd_batch_last_error",
-           "mlp_param_bytes", "mlp_init", "mlp_forward", "mlp_backward", "mlp_adam", "mhd_dump_faces",
+           "mlp_param_bytes", "mlp_init", "mlp_forward", "mlp_backward", "mlp_adam", "mlp_train_step", "mhd_dump_faces",
            "mhd_set_switch", "mhd_switch_choices", "mhd_measure_pipe_peaks", "mhd_stream_step",
            "mhd_stream_sync"]
 
@@ -168,6 +168,9 @@ def load(build: bool = True):
     L.mlp_backward.argtypes = [_VP, _VP, _VP, C.c_longlong, _VP, _VP]
     L.mlp_adam.restype = C.c_int
     L.mlp_adam.argtypes = [_VP, _VP, _VP, _VP, C.c_int, C.c_double, C.c_double, C.c_double, C.c_double, _VP]
+    L.mlp_train_step.restype = C.c_int
+    L.mlp_train_step.argtypes = [_VP, _VP, _VP, C.c_longlong, _VP, _VP, _VP, C.c_int, C.c_double, C.c_double,
+                                 C.c_double, C.c_double, _VP]
     L.mhd_dump_faces.restype = C.c_int
     L.mhd_dump_faces.argtypes = [_H, _VP, C.c_longlong, _VP, _VP, _VP]
     L.mhd_set_switch.restype = C.c_int
@@ -566,6 +569,12 @@ def mlp_backward(block_ptr, x_ptr, y_ptr, n, grad_ptr, stream=None):
 def mlp_adam(block_ptr, m_ptr, v_ptr, grad_ptr, step, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, stream=None):
     _rc(load().mlp_adam(_VP(block_ptr), _VP(m_ptr), _VP(v_ptr), _VP(grad_ptr), step, lr, beta1, beta2, eps,
                         _VP(stream or 0)), "mlp_adam")
+
+
+def mlp_train_step(block_ptr, x_ptr, y_ptr, n, grad_ptr, m_ptr, v_ptr, step, lr=1e-3, beta1=0.9, beta2=0.999,
+                   eps=1e-8, stream=None):
+    _rc(load().mlp_train_step(block_ptr, x_ptr, y_ptr, n, grad_ptr, m_ptr, v_ptr, step, lr, beta1, beta2, eps,
+                              stream or 0), "mlp_train_step")
 
 
 def mhd_dump_faces(h, ids_ptr, n, x_ptr, y_ptr, score_ptr=None):

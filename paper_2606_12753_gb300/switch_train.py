@@ -103,10 +103,9 @@ class Switch:
         return z
 
     def step(self, xb, yb, lr: float):
-        self.g.zero_()
-        mhd.mlp_backward(self.block.data_ptr(), xb.data_ptr(), yb.data_ptr(), xb.shape[0], self.g.data_ptr())
+        mhd.mlp_train_step(self.block.data_ptr(), xb.data_ptr(), yb.data_ptr(), xb.shape[0], self.g.data_ptr(),
+                           self.m.data_ptr(), self.v.data_ptr(), self.t + 1, lr=lr)
         self.t += 1
-        mhd.mlp_adam(self.block.data_ptr(), self.m.data_ptr(), self.v.data_ptr(), self.g.data_ptr(), self.t, lr=lr)
 
 
 def bce(z, y) -> float:

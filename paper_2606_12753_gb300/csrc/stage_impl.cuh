@@ -185,8 +185,8 @@ constexpr bool slopes_in_smem() {
 // own, each without the other's code.  A two-dimensional box in the kernel of
 // any box paid for the ring, the second copies of everything kept by plane
 // parity and one FP64 CTA per SM instead of two (HLL 3200^2 mixed, stage 1 / 2:
-// 1855 / 2066 us there, 1643 / 2014 here; Orszag-Tang 512^2 FP64: 794 / 841
-// and 632 / 679).
+// 1855 / 2066 us there, 1643 / 2014 here, 1246 / 1498 with four CTAs;
+// Orszag-Tang 512^2 FP64: 794 / 841 and 632 / 679).
 enum BoxKind { BOX_ANY = 0, BOX_3D = 1, BOX_2D = 2 };
 
 // Whether a kernel forms the slopes of the plane after next inside the flux
@@ -230,7 +230,7 @@ __host__ __device__ constexpr int ring_xo() {
 
 // Threads per CTA and CTAs per SM of the plain stage kernel: FP64 tiles run
 // 256 threads (1 CTA per SM, 2 for 8x8); the FP32-bulk forms keep 24 warps
-// per SM at about 85 registers a thread: 3 CTAs of 256 threads for tiles of up
+// per SM in 73 to 78 registers a thread: 3 CTAs of 256 threads for tiles of up
 // to 128 columns, 2 of 384 for 192 columns, 1 of 768 for 256 columns.
 template <int PREC, int TX, int TY>
 __host__ __device__ constexpr int stage_threads() {

@@ -1147,12 +1147,12 @@ __device__ __forceinline__ float cfl_bound(const Geo& g, float rho, const float 
 // difference, c_f,d^2 = (a^2 + b^2 + sqrt((a^2 - b^2)^2 + 4 a^2 b_t,d^2)) / 2.
 __device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double (&m)[3], double e,
                                           const double (&b)[3]) {
-  if (lt_(rho, g.rho_floor)) rho = g.rho_floor;
+  if (rho < g.rho_floor) rho = g.rho_floor;   // (not lt_: a cell with a NaN of either sign stays out of the maximum)
   const double ir = qrcp_(rho);
   const double b2[3] = {b[0] * b[0], b[1] * b[1], b[2] * b[2]};
   const double bb = b2[0] + b2[1] + b2[2];
   double p = g.gm1 * (e - 0.5 * (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) * ir - 0.5 * bb);
-  if (lt_(p, g.p_floor)) p = g.p_floor;
+  if (p < g.p_floor) p = g.p_floor;
   const double gp = g.gamma * p, a2 = gp * ir, q = bb * ir, x = a2 - q, s = a2 + q, xx = x * x, a4r = 4.0 * a2 * ir;
   double sum = 0.0;
 #pragma unroll
@@ -1225,19 +1225,20 @@ __global__ void __launch_bounds__(256) divb_kernel(Geo g, const S* U, unsigned l
   const int per_row = (g.n[0] + run - 1) / run;
   const long long items = (long long)g.n[1] * g.n[2] * per_row;
   const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
-  double m = 0.0;
+  long long m = 0;   // bits of the largest |div B|; non-negative doubles order as integers
   for (long long item = blockIdx.x * (long long)(blockDim.x / 32) + threadIdx.x / 32; item < items; item += nwarps) {
     const RowRun r = row_run(g, item, per_row, run);
     for (int i = r.i0 + lane; i < r.i1; i += 32) {
       const double div = (to_f64(U[r.x + (i + 1 < g.nf[0] ? i + 1 : 0)]) - to_f64(U[r.x + i])) * g.inv_d[0] +
                          (to_f64(U[r.yhi + i]) - to_f64(U[r.ylo + i])) * g.inv_d[1] +
                          (to_f64(U[r.zhi + i]) - to_f64(U[r.zlo + i])) * g.inv_d[2];
-      m = rmax(m, fabs(div));
+      const long long v = __double_as_longlong(fabs(div));
+      if (v <= 0x7ff0000000000000LL && v > m) m = v;   // cells that hold a NaN stay out
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = rmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0 && m > 0.0) atomicMax(word, (unsigned long long)__double_as_longlong(m));
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0 && m > 0) atomicMax(word, (unsigned long long)m);
 }
 
 static int reduce_word(mhd_handle* h, bool cfl, double* out) {

@@ -77,3 +77,22 @@ def test_cfl_dt(dims, bc, kind, precision):
     want = _dt(box)
     s.step(-1.0, 1)   # the last stage of the step before
     assert abs(s.stats()["last_dt"] / want - 1) <= fused
+
+
+@pytest.mark.parametrize("what", ["rho", "energy", "face"])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "fp32"])
+def test_reductions_leave_out_nan(what, sign, precision):
+    """Cells that hold a NaN of either sign, in the row of the maximum and elsewhere, stay out of both
+    maxima: the values of the state without them, exactly."""
+    box = I.random_state((37, 21, 40), seed=11)
+    box.cell[4][-1, -1, -1] *= 50.0      # the fastest cell
+    box.face[0][-1, -1, 34] += 3.0       # the largest |div B|, in its row
+    s = mhd.Solver(box, precision=precision)
+    s.set_state(box.cell, box.face)
+    want = s.cfl_dt(), s.divb_max()
+    nan = np.copysign(np.nan, sign)
+    for at in ((-1, -1, 8), (3, 4, 5), (20, 0, 36)):
+        (box.cell[0] if what == "rho" else box.cell[4] if what == "energy" else box.face[1])[at] = nan
+    s.set_state(box.cell, box.face)
+    assert (s.cfl_dt(), s.divb_max()) == want

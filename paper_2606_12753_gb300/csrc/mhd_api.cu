@@ -303,40 +303,42 @@ static MarchRates march_rates(bool fp64, int most) {
   return {most, {{1.0}, {0.90, 0.75}, {0.825, 0.67, 0.515}}, 1.65};
 }
 
-static double march_time(std::vector<ChunkGroup> groups, const MarchRates& m) {
+// (`groups` is used up.  No heap: a step of mhd_step_noalloc comes here.)
+static double march_time(ChunkGroup* groups, size_t ngroups, const MarchRates& m) {
   struct SMs {
     int count, n;
     double left[3];   // of the resident chunks, oldest first
   };
-  std::vector<SMs> sms{{kSMs, 0, {}}}, merged;
+  SMs sms[kSMs], merged[kSMs];   // every entry stands for at least one SM
+  int nsms = 1;
+  sms[0] = {kSMs, 0, {}};
   double time = 0.0;
   size_t next = 0;
   for (int event = 0; event < 1 << 14; ++event) {
     for (int n = 0; n < m.most; ++n)   // waiting chunks go to the emptiest SMs first
-      for (size_t i = 0; i < sms.size(); ++i) {
-        while (next < groups.size() && groups[next].count == 0) ++next;
-        if (next == groups.size()) break;
+      for (int i = 0; i < nsms; ++i) {
+        while (next < ngroups && groups[next].count == 0) ++next;
+        if (next == ngroups) break;
         if (sms[i].n != n) continue;
         const int take = (int)std::min<long long>(sms[i].count, groups[next].count);
         if (take < sms[i].count) {
-          SMs rest = sms[i];
-          rest.count -= take;
+          sms[nsms] = sms[i];
+          sms[nsms++].count -= take;
           sms[i].count = take;
-          sms.push_back(rest);
         }
         sms[i].left[sms[i].n++] = groups[next].planes + m.prologue;
         groups[next].count -= take;
       }
     double step = HUGE_VAL;
-    for (const SMs& c : sms)
-      for (int i = 0; i < c.n; ++i) step = std::min(step, c.left[i] / m.rate[c.n - 1][i]);
+    for (int c = 0; c < nsms; ++c)
+      for (int i = 0; i < sms[c].n; ++i) step = std::min(step, sms[c].left[i] / m.rate[sms[c].n - 1][i]);
     if (step == HUGE_VAL) return time;
     time += step;
-    merged.clear();
-    for (const SMs& c : sms) {
-      SMs d = {c.count, 0, {}};
-      for (int i = 0; i < c.n; ++i) {
-        const double left = c.left[i] - step * m.rate[c.n - 1][i];
+    int nmerged = 0;
+    for (int c = 0; c < nsms; ++c) {
+      SMs d = {sms[c].count, 0, {}};
+      for (int i = 0; i < sms[c].n; ++i) {
+        const double left = sms[c].left[i] - step * m.rate[sms[c].n - 1][i];
         if (left > 1e-6) d.left[d.n++] = left;
       }
       const auto alike = [&](const SMs& e) {
@@ -345,11 +347,13 @@ static double march_time(std::vector<ChunkGroup> groups, const MarchRates& m) {
           if (std::fabs(e.left[i] - d.left[i]) > 1e-4) return false;
         return true;
       };
-      const auto it = std::find_if(merged.begin(), merged.end(), alike);
-      if (it == merged.end()) merged.push_back(d);
+      SMs* const end = merged + nmerged;
+      SMs* const it = std::find_if(merged, end, alike);
+      if (it == end) merged[nmerged++] = d;
       else it->count += d.count;
     }
-    sms.swap(merged);
+    std::copy(merged, merged + nmerged, sms);
+    nsms = nmerged;
   }
   return HUGE_VAL;
 }
@@ -376,10 +380,8 @@ static int default_chunk(const mhd_config* c, int tx, int ty) {
   const MarchRates rates = march_rates(c->precision == MHD_FP64, resident_ctas(c, tx, ty));
   const auto estimate = [&](int tz) {
     const int n = (c->nz + tz - 1) / tz, last = c->nz - (n - 1) * tz;
-    std::vector<ChunkGroup> groups;
-    if (n > 1) groups.push_back({tz, columns * (n - 1)});
-    groups.push_back({last, columns});
-    return march_time(groups, rates);
+    ChunkGroup groups[2] = {{tz, columns * (n - 1)}, {last, columns}};
+    return march_time(groups, 2, rates);
   };
   int best = 32;
   const double base = estimate(32);
@@ -1429,7 +1431,7 @@ static int batch_default_chunk(const mhd_batch* b, int tx, int ty) {
     if (tz < 16 && items > 40LL * kSMs * rates.most) continue;
     std::vector<ChunkGroup> groups;
     for (const auto& q : count) groups.push_back({q.first, q.second});
-    const double t = march_time(groups, rates);
+    const double t = march_time(groups.data(), groups.size(), rates);
     if (tz == 32) least = 0.98 * t;
     else if (t < least) {
       least = t;

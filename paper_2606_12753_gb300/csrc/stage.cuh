@@ -313,20 +313,43 @@ __device__ __forceinline__ float cut32(double x) {
   return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), hi, 3) - (896u << 23));
 }
 
+// Sum over the active axes of (|v_d| + c_f,d) / Delta_d from |v_d|, the sound
+// speed a^2 and b_d^2 = B_d^2 / rho: c_f,d^2 = (a^2 + b^2 + sqrt((a^2 - b^2)^2 +
+// 4 a^2 (b^2 - b_d^2))) / 2, whose terms only add: nothing cancels, and a term
+// that overflows makes the sum infinite or NaN, never smaller.
+template <typename R>
+__device__ __forceinline__ R signal_sum(const Geo& g, const R (&v)[3], R a2, const R (&b2)[3]) {
+  const R bb = b2[0] + b2[1] + b2[2], x = a2 - bb, s = a2 + bb, xx = x * x, a4 = R(4) * a2;
+  R sum = R(0);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    if (g.n[d] > 1) {
+      const R root = qroot_(xx + a4 * (b2[(d + 1) % 3] + b2[(d + 2) % 3]));
+      sum += (v[d] + qroot_(R(0.5) * (s + root))) * gpar<R>(g.inv_d[d], g.finv_d[d]);
+    }
+  }
+  return sum;
+}
+
 // Whether a cell's CFL speed sum may exceed `top` (positive): its value in
-// FP32, which is off by less than 1e-3 (inputs cut by 2^-23, and the
-// root of a difference that cancels loses half of FP32's digits), against
-// top.  A CFL maximum is of its start's order after a few cells, so nearly
-// every cell is settled by ~50 FP32 instructions instead of ~75 FP64 ones,
-// each of which holds the FP64 pipe for ~17 cycles (128^3 FP64, last stage:
-// 5826 -> 5450 us).  Pressures and densities
-// near the ends of FP32's range, and NaN, answer yes.
+// FP32, which is off by less than 1e-5 (inputs cut by 2^-23, a few roundings
+// of terms that only add), against top.  A CFL maximum is of its start's order
+// after a few cells, so nearly every cell is settled by ~50 FP32 instructions
+// instead of ~75 FP64 ones, each of which holds the FP64 pipe for ~17 cycles.
+// Yes is the answer where FP32's range could make the value too small:
+// densities and pressures near its ends, sound speeds below 1e-8 (whose fourth
+// powers underflow; fields that underflow are far below such a sound speed),
+// sums near its lower end (cells of 1e38 across), and to NaN.  Overflow makes
+// the value infinite or NaN.
 __device__ __forceinline__ bool cfl_may_exceed(const Geo& g, const double* w, double top) {
   float f[8];
 #pragma unroll
   for (int v = 0; v < 8; ++v) f[v] = cut32(fabs(w[v]));
-  if (!(f[0] > 1e-30f && f[0] < 1e30f && f[4] > 1e-30f && f[4] < 1e30f)) return true;
-  return !(cfl_speed<float>(g, f) * 1.002f < cut32(top));
+  const float ir = 1.0f / f[0], a2 = g.fgamma * f[4] * ir;
+  if (!(f[0] > 1e-30f && f[0] < 1e30f && f[4] > 1e-30f && f[4] < 1e30f && a2 > 1e-16f)) return true;
+  const float v[3] = {f[1], f[2], f[3]}, b2[3] = {f[5] * f[5] * ir, f[6] * f[6] * ir, f[7] * f[7] * ir};
+  const float sum = signal_sum(g, v, a2, b2);
+  return !(sum > 1e-30f && sum * 1.002f < cut32(top));
 }
 
 // Whether a recovered cell holds a value that is not finite (as the sums of

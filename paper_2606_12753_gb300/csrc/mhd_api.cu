@@ -1113,36 +1113,32 @@ __device__ __forceinline__ float signed32(double x) { return copysignf(cut32(fab
 // more than their rounding (1e-6 of the terms they are formed from; p
 // subtracts the field at its lower end), and the rest is a few roundings (the
 // factor at the end).  Infinity where FP32's exponent range does not hold the
-// terms.
+// terms: energies near its end (a pressure formed from infinities could drop
+// to its floor), densities and pressures near its ends, sound speeds below
+// 1e-8 (whose fourth powers underflow), sums near its lower end (cells of 1e38
+// across).  Fields that overflow make the sum infinite or NaN by themselves.
 __device__ __forceinline__ float cfl_bound(const Geo& g, float rho, const float (&m)[3], float e, const float (&lo)[3],
                                            const float (&hi)[3]) {
   const float inf = __int_as_float(0x7f800000);
   rho = fmaxf(rho, g.frho_floor);
   const float ir = 1.0f / rho;
-  float b[3], mm = 0.f, bb = 0.f, bl = 0.f;
+  float v[3], b2[3], mm = 0.f, bl = 0.f;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float c = 0.5f * fabsf(lo[d] + hi[d]), err = 1e-6f * (fabsf(lo[d]) + fabsf(hi[d]));
-    const float low = fmaxf(c - err, 0.f);
-    b[d] = c + err;
+    const float low = fmaxf(c - err, 0.f), high = c + err;
+    v[d] = m[d] * ir;
+    b2[d] = high * high * ir;
     mm += m[d] * m[d];
-    bb += b[d] * b[d];
     bl += low * low;
   }
-  const float kin = 0.5f * mm * ir, mag = 0.5f * bl;
-  float p = g.fgm1 * (fabsf(e) * 1.000001f - kin - mag + 4e-6f * (fabsf(e) + kin + mag));
+  const float kin = 0.5f * mm * ir, mag = 0.5f * bl, terms = fabsf(e) + kin + mag;
+  float p = g.fgm1 * (fabsf(e) * 1.000001f - kin - mag + 4e-6f * terms);
   p = fmaxf(p, g.fp_floor * 1.000001f);
-  const float a2 = g.fgamma * p * ir, b2 = bb * ir, x = a2 - b2;
-  if (!(rho > 1e-30f && rho < 1e30f && p > 1e-30f && p < 1e30f && a2 > 1e-18f && a2 < 1e18f)) return inf;
-  float sum = 0.f;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    if (g.n[d] > 1) {
-      const float root = sqrtf(x * x + 4.0f * a2 * (b2 - b[d] * b[d] * ir * 0.999999f));
-      sum += (m[d] * ir + sqrtf(0.5f * (a2 + b2 + root))) * g.finv_d[d];
-    }
-  }
-  return sum * 1.00001f;
+  const float a2 = g.fgamma * p * ir;
+  if (!(terms < 1e37f && rho > 1e-30f && rho < 1e30f && p > 1e-30f && p < 1e30f && a2 > 1e-16f)) return inf;
+  const float sum = signal_sum(g, v, a2, b2);
+  return sum > 1e-30f ? sum * 1.00001f : inf;
 }
 
 // The speed sum in FP64: the three fast speeds share a^2, b^2 and their

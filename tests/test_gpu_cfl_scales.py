@@ -1,8 +1,9 @@
 """The CFL maximum in units far from one.  The cells that need no FP64 speed
 are found by an FP32 estimate, whose squares leave binary32's range at speeds
 of about 1e10 and of 1e-10: the dt of the fused FP64 step, of a box of a batch
-and of the allocation-free step must still be cfl over the largest FP64 speed.  The fastest cell, 2 % above most others, lies
-late in every march and row.  Tolerance: 40 roundings (1e-14) times the
+and of the allocation-free step, and that of the standalone reduction of every
+form, must still be cfl over the largest FP64 speed.  The fastest cell, 2 %
+above most others, lies late in every march and row.  Tolerance: 40 roundings (1e-14) times the
 energy over the thermal energy (below 10)."""
 import numpy as np
 import pytest
@@ -104,3 +105,24 @@ def test_allocation_free_step(scale):
     dt = mhd.mhd_step_noalloc(cfg, [c.data_ptr() for c in cell], [f.data_ptr() for f in face],
                               [c.data_ptr() for c in oc], [f.data_ptr() for f in of], -1.0)
     assert abs(dt / want - 1) <= 1e-14
+
+
+# the standalone reduction, whose FP32 bound subtracts energies: rho, speed, p, pressure floor; the last three hold
+# momenta whose squares leave binary32's range, and floors that a pressure lost in infinities would fall to
+BOUND = {"fast": (1.0, 1e10, 6e19, 1e10), "slow": (1.0, 1e-12, 6e-25, 1e-33), "heavy": (1e20, 1e5, 6e29, 1e20),
+         "dense, fast": (1e14, 1e9, 1e32, 1e10), "dense, slow": (1e25, 1e-3, 1e24, 1e10),
+         "supersonic": (1e14, 1e9, 1e28, 1e12)}
+
+
+@pytest.mark.parametrize("scale", BOUND)
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "fp32"])
+def test_reduction(scale, precision):
+    rho, speed, p, floor = BOUND[scale]
+    box = _box((64, 100, 100), rho, speed, 1e-3)
+    box.cell[4] += (p - 0.6 * rho * speed ** 2) / (box.gamma - 1)
+    s = mhd.Solver(box, precision=precision, p_floor=floor)
+    s.set_state(box.cell, box.face)
+    cell, face = s.get_state()   # rounded to the form's state
+    box.cell, box.face = cell.astype(np.float64), [f.astype(np.float64) for f in face]
+    amplified = max(1.0, (box.cell[4] * (box.gamma - 1) / p).max() / 10.0)
+    assert abs(s.cfl_dt() / _dt(box) - 1) <= 1e-14 * amplified

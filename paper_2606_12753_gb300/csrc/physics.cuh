@@ -110,16 +110,34 @@ __host__ __device__ __forceinline__ double rsqrt_(double x) {   // square root
 }
 // The same three with fewer FP64-pipe operations again (rcp 2, rsqrt and root
 // 3), where the result may round differently (the characteristic slopes and
-// the lean solvers below).  With the residual e of the seed y the result is
-// y (1 + e + e^2) (rcp), y (1 + e/2 + 3/8 e^2) (the roots); the last term,
-// ~1e-12 of y, is formed in FP32 and added to y's bits as an integer number of
-// ulps, and the step to the result is one fma.  Halving is an exponent
-// decrement.  A face has nine of them: 128^3 HLLD 4787 / 4900 -> 4573 / 4676 us.
-// (Adding e^2 to e's own bits instead is exact to fewer ulps but needs a test
-// for the next binade, which cost more than the operations it saved.)
+// the lean solvers below), and no less exact.  With the residual e of the seed
+// y (t = x y for the root) the result is y + y (1 + e) e (rcp), y + y/2 (1 +
+// 3/4 e) e (rsqrt), t (1 + 3/8 e^2) + t/2 e (root).  What stands before the
+// last e is needed to 2^-33 only: it is formed on the bits of y, and the step
+// to the result is one fma.  Halving is an exponent decrement.  A face has
+// nine of them.  Errors in ulps, largest / mean of random mantissas: rcp 0.507 /
+// 0.250, rsqrt 0.999 / 0.276, root 1.25 / 0.352; the forms above 0.508 / 0.250,
+// 0.999 / 0.276, 1.73 / 0.383.  (Steps on the bits of e, or of y for any y, need a
+// test for the next binade: 128^3 HLLD 6 % slower than these.)
 #ifdef __CUDA_ARCH__
-// y (1 + (EIGHTHS / 8) e^2), y normal, |e| < 1e-4 (half an ulp from rounding; a
-// step into the next binade, one in 10^12, is off by at most the step)
+// y (1 + (EIGHTHS / 8) e) to 2^-40 of itself, for a hardware seed y (20 leading
+// mantissa bits, the others zero) and its residual, |e| < 2^-19.8: e times y's
+// mantissa, in FP32 (e below 2^-62 counts as that), as a number of 2^12 ulps (the
+// integer in the low bits of a float of 1.5 x 2^23) added to y's bits.  Below a
+// mantissa of 1.0 an ulp is half of one; no seed is closer to 2.0 than its e.
+template <int EIGHTHS>
+__device__ __forceinline__ double scaled_seed(double y, double e) {
+  constexpr float kUnit = 0.125f * EIGHTHS * 1099511627776.0f;   // in 2^12 ulps of [1, 2)
+  const unsigned my = ((unsigned)__double2hiint(y) << 3 & 0x007fffffu) | 0x3f800000u;
+  const float up = __uint_as_float(my) * kUnit, down = my == 0x3f800000u ? 2.0f * kUnit : up;
+  const int he = __double2hiint(e);
+  const unsigned mag = max((unsigned)he & 0x7fffffffu, 0x3c100000u);
+  const float step = fmaf(__uint_as_float((mag << 3) - (896u << 23)), he < 0 ? -down : up, 12582912.0f);
+  return __longlong_as_double(__double_as_longlong(y) + (long long)(__float_as_int(step) - 0x4b400000) * 4096);
+}
+// y (1 + (EIGHTHS / 8) e^2), y normal, |e| < 1e-4, half an ulp from rounding: the
+// last term, formed in FP32, as a number of ulps (a step into the next
+// binade, one in 10^12, is off by at most the step)
 template <int EIGHTHS>
 __device__ __forceinline__ double plus_square(double y, double e) {
   const unsigned he = (unsigned)__double2hiint(e) & 0x7fffffffu;
@@ -139,7 +157,7 @@ __host__ __device__ __forceinline__ double qrcp_(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x, r, 1.0);
-  return fma(r, e, plus_square<8>(r, e));
+  return fma(scaled_seed<8>(r, e), e, r);
 #else
   return 1.0 / x;
 #endif
@@ -150,7 +168,7 @@ __host__ __device__ __forceinline__ double qrsqrt_(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-(x * y), y, 1.0);
-  return fma(half_(y), e, plus_square<3>(y, e));
+  return fma(scaled_seed<6>(half_(y), e), e, y);
 #else
   return 1.0 / sqrt(x);
 #endif

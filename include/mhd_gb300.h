@@ -355,10 +355,11 @@ int mhd_batch_step_async(mhd_batch* b, double dt, int nsteps);
  * kernel; get also returns the number of work items and the persistent grid. */
 int mhd_batch_set_tile(mhd_batch* b, int tx, int ty, int tz);
 int mhd_batch_get_tile(mhd_batch* b, int tile[3], long long* items, int* grid);
-/* Time every instantiated tile shape and z-chunk length for trial_steps
- * steps on this batch (the states are restored afterwards), keep the fastest
- * and append it to the JSON-lines cache at cache_path (NULL: no cache), keyed
- * by device, precision, Riemann solver and the box sizes; a cached key is
+/* Time the current tile and every instantiated tile shape, at its default
+ * z-chunk length and a few fixed ones, for trial_steps steps on this batch
+ * (the states are restored afterwards), keep the fastest and append it to the
+ * JSON-lines cache at cache_path (NULL: no cache), keyed by device, precision,
+ * Riemann solver, the box sizes and the set of lengths; a cached key is
  * applied without trials.  tile_out / ms_out (may be NULL) receive the choice
  * and its time per step. */
 int mhd_batch_autotune(mhd_batch* b, int trial_steps, const char* cache_path, int tile_out[3], double* ms_out);

@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <functional>
 #include <map>
 #include <new>
@@ -1816,10 +1817,11 @@ extern "C" int mhd_batch_get_stats(mhd_batch* b, mhd_stats* out) {
 }
 
 // ---------------------------------------------------------------- autotuner
-// Times every instantiated tile shape (and a few z-chunk lengths) on the
-// batch itself for `trial_steps` steps, keeps the fastest, and records it in
-// a JSON-lines cache keyed by device, precision, Riemann solver and the box
-// sizes, so later runs on the same batch skip the trials.
+// Times the tile the batch has and every instantiated tile shape (at its
+// default z-chunk length and a few fixed ones) on the batch itself for
+// `trial_steps` steps, keeps the fastest, and records it in a JSON-lines cache
+// keyed by device, precision, Riemann solver, the box sizes and the set of
+// lengths tried, so later runs on the same batch skip the trials.
 
 static std::string batch_key(mhd_batch* b) {
   int dev = 0, maj = 0, min = 0;
@@ -1834,7 +1836,7 @@ static std::string batch_key(mhd_batch* b) {
     cells += (long long)n[0] * n[1] * n[2];
   }
   char buf[256];
-  snprintf(buf, sizeof buf, "sm_%d%d|prec%d|riemann%d|nbox%d|cells%lld|dims%016llx", maj, min, b->prec,
+  snprintf(buf, sizeof buf, "sm_%d%d|prec%d|riemann%d|nbox%d|cells%lld|dims%016llx|z2", maj, min, b->prec,
            b->cfg[0].riemann, b->nbox, cells, h);
   return buf;
 }
@@ -1892,32 +1894,38 @@ extern "C" int mhd_batch_autotune(mhd_batch* b, int trial_steps, const char* cac
   static const int cand_z[] = {16, 32, 64, 128};
   int maxnz = 1;
   for (int i = 0; i < b->nbox; ++i) maxnz = b->cfg[i].nz > maxnz ? b->cfg[i].nz : maxnz;
+  // the batch's own tile first; a shape's default length only where it is none of the fixed ones
+  std::vector<std::array<int, 3>> cand = {{b->tx, b->ty, b->tz}};
+  const auto propose = [&](int tx, int ty, int tz) {
+    const std::array<int, 3> t = {tx, ty, tz};
+    if (std::find(cand.begin(), cand.end(), t) == cand.end()) cand.push_back(t);
+  };
+  for (const auto& xy : cand_xy) {
+    for (int zi = 0; zi < 4 && (zi == 0 || cand_z[zi - 1] < maxnz); ++zi) propose(xy[0], xy[1], cand_z[zi]);
+    propose(xy[0], xy[1], batch_default_chunk(b, xy[0], xy[1]));
+  }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   best_ms = -1.0;
-  for (const auto& xy : cand_xy) {
-    for (int zi = 0; zi < 4; ++zi) {
-      const int tz = cand_z[zi];
-      if (zi > 0 && cand_z[zi - 1] >= maxnz) break;
-      if (batch_apply_tile(b, xy[0], xy[1], tz) != MHD_OK) break;   // tile not instantiated
-      if (batch_enqueue(b, -1.0, 1) != MHD_OK) continue;
-      cudaEventRecord(e0, b->stream);
-      if (batch_enqueue(b, -1.0, trial_steps) != MHD_OK) continue;
-      cudaEventRecord(e1, b->stream);
-      if (batch_check(b) != MHD_OK) continue;
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      const double per = ms / trial_steps;
-      if (best_ms < 0.0 || per < best_ms) {
-        best_ms = per;
-        best[0] = xy[0]; best[1] = xy[1]; best[2] = tz;
-      }
-      // restore the states for the next candidate
-      for (int i = 0; i < b->nbox; ++i) {
-        cudaMemcpyAsync(b->box[i].U[b->box[i].cur], save[i], b->ubytes[i], cudaMemcpyDeviceToDevice, b->stream);
-        b->prims_valid[i] = false;
-      }
+  for (const auto& t : cand) {
+    if (batch_apply_tile(b, t[0], t[1], t[2]) != MHD_OK) continue;   // tile not instantiated
+    if (batch_enqueue(b, -1.0, 1) != MHD_OK) continue;
+    cudaEventRecord(e0, b->stream);
+    if (batch_enqueue(b, -1.0, trial_steps) != MHD_OK) continue;
+    cudaEventRecord(e1, b->stream);
+    if (batch_check(b) != MHD_OK) continue;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    const double per = ms / trial_steps;
+    if (best_ms < 0.0 || per < best_ms) {
+      best_ms = per;
+      best[0] = t[0]; best[1] = t[1]; best[2] = t[2];
+    }
+    // restore the states for the next candidate
+    for (int i = 0; i < b->nbox; ++i) {
+      cudaMemcpyAsync(b->box[i].U[b->box[i].cur], save[i], b->ubytes[i], cudaMemcpyDeviceToDevice, b->stream);
+      b->prims_valid[i] = false;
     }
   }
   cudaEventDestroy(e0);

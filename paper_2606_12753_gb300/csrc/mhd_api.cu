@@ -685,17 +685,36 @@ __global__ void __launch_bounds__(256) state_copy_kernel(StateCopy c) {
   else copy_as<unsigned>(c.src[q], c.dst[q], c.bytes[q]);
 }
 
-// Whether p is plain memory of the current device (anything else, a host
-// pointer passed for a device one among it, goes to the runtime's copy).
-static bool device_memory(const void* p) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+// How the bytes from p on may be copied: by the kernel where they are plain
+// memory of the current device, by the runtime's copy where they are anything
+// else (a host pointer passed for a device one among it); not at all where they
+// run past the end of the cudaMalloc allocation that p lies in, which the
+// runtime's copy refuses and a kernel would not notice.  (Of memory mapped
+// piecewise the driver knows the piece; the runtime's copy judges that.)
+enum CopyKind { COPY_KERNEL, COPY_RUNTIME, COPY_REFUSED };
+static CopyKind copy_kind(const void* p, unsigned long long bytes, int current) {
+  static const auto attributes = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
     cudaGetLastError();
-    return false;
-  }
-  int dev = -1;
-  return at.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && at.device == dev &&
-         ((uintptr_t)p & 3) == 0;
+    return (CUresult(*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr))f;
+  }();
+  unsigned type = 0, managed = 0, whole = 0;
+  int device = -1;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute ask[6] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,     CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE,      CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE};
+  void* out[6] = {&type, &managed, &device, &start, &size, &whole};
+  const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+  if (!attributes || attributes(6, ask, out, at) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed)
+    return COPY_RUNTIME;
+  if (at < start || at - start > size || bytes > size - (at - start)) return whole ? COPY_REFUSED : COPY_RUNTIME;
+  return device == current && (at & 3) == 0 ? COPY_KERNEL : COPY_RUNTIME;
 }
 
 namespace mhd {
@@ -703,7 +722,10 @@ namespace mhd {
 cudaError_t copy_state_on_device(const Geo& g, bool in, char* base, size_t elem, void* const* cell, void* const* face,
                                  cudaStream_t st) {
   StateCopy c;
-  bool plain = true;
+  int current = -1;
+  cudaError_t e = cudaGetDevice(&current);
+  if (e != cudaSuccess) return e;
+  bool plain = copy_kind(base, 0, current) == COPY_KERNEL;   // (a handle of another device than the current one)
   unsigned long long most = 0;
   for (int q = 0; q < 8; ++q) {
     void* user = q < 5 ? cell[q] : face[q - 5];
@@ -712,14 +734,15 @@ cudaError_t copy_state_on_device(const Geo& g, bool in, char* base, size_t elem,
     c.dst[q] = in ? own : user;
     c.bytes[q] = (unsigned long long)(q < 5 ? g.ncell : face_count(g, q - 5)) * elem;
     most = std::max(most, c.bytes[q]);
-    plain = plain && device_memory(user);
+    const CopyKind kind = copy_kind(user, c.bytes[q], current);
+    if (kind == COPY_REFUSED) return cudaErrorInvalidValue;
+    plain = plain && kind == COPY_KERNEL;
   }
   if (plain) {
     const unsigned blocks = (unsigned)std::min<unsigned long long>((most + 4095) / 4096, 152ull * 4);
     state_copy_kernel<<<dim3(blocks, 8), 256, 0, st>>>(c);
     return cudaGetLastError();
   }
-  cudaError_t e = cudaSuccess;
   for (int q = 0; q < 8 && e == cudaSuccess; ++q)
     e = cudaMemcpyAsync(c.dst[q], c.src[q], c.bytes[q], cudaMemcpyDeviceToDevice, st);
   return e;

@@ -474,8 +474,12 @@ struct StageKernel {
   }
 
   // The Riemann solvers of this form (physics.cuh): the ones of fewer
-  // operations in FP64, but for a two-dimensional box, whose out-of-plane
-  // field may be rounding alone.
+  // operations in FP64, but for the kernels of a single two-dimensional box,
+  // whose out-of-plane field may be rounding alone.  A two-dimensional FP64 box
+  // of a batch, with the learned switch or characteristic reconstruction takes
+  // the shorter ones, as every box of those kernels: its states are the single
+  // box's to rounding only (Orszag-Tang 64^2, ten steps: 4e-15), and the
+  // out-of-plane field of a planar flow, 1e-17 there, stays zero here.
   static constexpr bool kLean = PREC == P_FP64 && !FLAT;
   static __device__ __forceinline__ void solve_hll(const R* wl, const R* wr, R bn, R gam, R ig, R* f, R* cm) {
     if constexpr (kLean) hll_flux_lean(wl, wr, bn, gam, ig, f, cm);

@@ -280,7 +280,7 @@ extern "C" void mhd_default_config(mhd_config* c, int nx, int ny, int nz) {
 // the next chunk when one of its own ends.  The CTAs of an SM do not share it
 // evenly: the one that started first issues first and runs ahead, so that a
 // launch of one wave ends with its SMs half empty (mixed 240^3: 240 planes a
-// chunk 2304 us a stage, 32 planes 2042).  rate[n - 1] holds the planes per
+// chunk 2237 us a stage, 32 planes 1969).  rate[n - 1] holds the planes per
 // unit of an SM's n CTAs, oldest first.  A chunk costs its planes and a
 // prologue.  SMs in the same state advance together.
 struct ChunkGroup {
@@ -368,10 +368,10 @@ static int resident_ctas(const mhd_config* c, int tx, int ty) {
 
 // Default planes per z-chunk: 32, unless march_time finds a length that takes
 // less than 0.98 of it.  Small boxes then have chunks enough for every SM (us a
-// stage: 24^3 FP64 1 plane a chunk 112, one chunk of 24 989; 64^3 mixed 5: 68,
-// 32: 186) and middle ones no nearly empty last wave (128^3 FP64 16: 4713, 32:
-// 5094; 128^3 mixed 15: 377, 32: 461; 97x130x75 FP32 13: 210, 32: 240; 240^3
-// mixed stays at 32: 2048, one chunk of 240: 2306).  On 17 sizes from 24^3 to
+// stage: 24^3 FP64 1 plane a chunk 109, one chunk of 24 975; 64^3 mixed 5: 66,
+// 32: 181) and middle ones no nearly empty last wave (128^3 FP64 16: 4619, 32:
+// 5001; 128^3 mixed 15: 362, 32: 437; 97x130x75 FP32 13: 204, 32: 236; 240^3
+// mixed stays at 32: 1969, one chunk of 240: 2237).  On 17 sizes from 24^3 to
 // 352^3 and all precisions the choice took at most 1.7 % more than the best length.
 // Results do not depend on it, but for the learned switch in FP32 arithmetic,
 // whose first pass over a chunk rounds differently: it keeps 32.
@@ -1165,7 +1165,8 @@ __device__ __forceinline__ float cfl_bound(const Geo& g, float rho, const float 
   return sum > 1e-30f ? sum * 1.00001f : inf;
 }
 
-// The speed sum in FP64: the three fast speeds share a^2, b^2 and their
+// The speed sum in FP64 (signal_sum from conserved values, with the division
+// by rho taken out of the roots): the three fast speeds share a^2, b^2 and their
 // difference, c_f,d^2 = (a^2 + b^2 + sqrt((a^2 - b^2)^2 + 4 a^2 b_t,d^2)) / 2.
 __device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double (&m)[3], double e,
                                           const double (&b)[3]) {
@@ -1190,8 +1191,8 @@ __device__ __forceinline__ double cfl_sum(const Geo& g, double rho, const double
 // CFL maximum.  The FP64 sum (~70 operations of a pipe that takes ~17 cycles
 // for each) is formed only by warps with a cell whose FP32 bound is not below
 // the largest sum found so far, which every warp reads before a run.
-// Measured (GB300): 256^3 mixed 464 us (4742 with every sum in FP64 and
-// IEEE divides), 97x130x75 FP32 139 (424).
+// Measured (GB300), a call with its synchronisation: 256^3 mixed 480 us (4742 with
+// every sum in FP64 and IEEE divides), 97x130x75 FP32 68 (424).
 template <typename S>
 __global__ void __launch_bounds__(256) cfl_kernel(Geo g, const S* U, unsigned long long* word, int run) {
   const int lane = threadIdx.x & 31;

@@ -117,8 +117,10 @@ __host__ __device__ __forceinline__ double rsqrt_(double x) {   // square root
 // to the result is one fma.  Halving is an exponent decrement.  A face has
 // nine of them.  Errors in ulps, largest / mean of random mantissas: rcp 0.507 /
 // 0.250, rsqrt 0.999 / 0.276, root 1.25 / 0.352; the forms above 0.508 / 0.250,
-// 0.999 / 0.276, 1.73 / 0.383.  (Steps on the bits of e, or of y for any y, need a
-// test for the next binade: 128^3 HLLD 6 % slower than these.)
+// 0.999 / 0.276, 1.73 / 0.383.  Measured (GB300, stage 1 / 2): 128^3 HLLD 4887 /
+// 4976 us with the forms above, 4619 / 4717 with these, HLL 4432 / 4505 and 4286 /
+// 4355, characteristic 96x64x80 1983 / 1976 and 1843 / 1837.  (Steps on the bits
+// of e, or of y for any y, need a test for the next binade: 128^3 6 % slower.)
 #ifdef __CUDA_ARCH__
 // y (1 + (EIGHTHS / 8) e) to 2^-40 of itself, for a hardware seed y (20 leading
 // mantissa bits, the others zero) and its residual, |e| < 2^-19.8: e times y's
@@ -460,13 +462,13 @@ __host__ __device__ __forceinline__ void hlld_flux(const R* wl, const R* wr, R b
 // ---------------------------------------------------------------------------
 // The same two solvers with fewer operations: the forms of the FP64 kernels,
 // which are bound by the FP64 pipe (one warp-instruction per ~17 SM cycles,
-// the other pipes nearly idle).  They equal the forms above up to rounding
-// and are the nearer ones to the exact flux (random faces against 80-bit
-// arithmetic: HLLD 2.6e-17 of the flux scale on the mean against 6.1e-17,
-// HLL 2.2e-17 against 2.4e-17).  FP32 fluxes keep the forms above: a change
-// of FP32 rounding flips limiter and upwind choices here and there, which
-// moves single cells by 1e-3.  Per face an HLLD solution takes about 160 FP64
-// operations instead of 250, by these identities:
+// the other pipes nearly idle).  They equal the forms above up to rounding,
+// times the conditioning of the star states.  FP32 fluxes keep the forms above:
+// a change of FP32 rounding flips limiter and upwind choices here and there,
+// which moves single cells by 1e-3.  As written, an HLLD solution takes 59
+// additions and 85 multiplications instead of 107 and 169 (mean of random
+// faces, fused ones counted apart; HLL 66 and 93 instead of 80 and 142), and
+// fewer roots and reciprocals, by these identities:
 //   * c_f^2 = T / (2 rho), T = gamma p + |B|^2 + sqrt((gamma p - |B|^2)^2 + 4 gamma p |B_t|^2):
 //     the larger of two fast speeds is found by comparing T_L rho_R with
 //     T_R rho_L, and one division and one outer root serve both states;
@@ -478,8 +480,8 @@ __host__ __device__ __forceinline__ void hlld_flux(const R* wl, const R* wr, R b
 //   * across an Alfven wave v** - v* = +-sgn(bn) (B** - B*)/sqrt(rho*);
 //   * only the side of S_M that holds the face forms its energy, and the
 //     other side's star state is formed only where a double-star state needs it.
-// Measured (GB300, 128^3, stage 1 / 2 in us): HLLD 7197 / 7678 with the plain
-// solvers, 5521 / 5984 with these; HLL 5487 / 5967 and 5031 / 5515.
+// Measured (GB300, 128^3, stage 1 / 2 in us): HLLD 6389 / 6480 with the plain
+// solvers, 4619 / 4717 with these; HLL 4837 / 4901 and 4286 / 4355.
 
 // The larger fast speed of two states, b2_* = |B|^2 and bt2_* = |B_t|^2 of each.
 __host__ __device__ __forceinline__ double max_fast_speed(const double* wl, const double* wr, double b2_l, double b2_r,
@@ -694,9 +696,9 @@ __host__ __device__ __forceinline__ R upwind_nz(R m, R lo_a, R lo_b, R hi_a, R h
 // exactly zero is rare (rest, or inside the deadband), so FP64 forms the mean
 // it asks for only where one of the four is: four differences instead of
 // eight and no means, half of an edge's FP64 operations (128^3, stage 1 / 2:
-// 5525 / 5981 -> 5374 / 5826 us).  FP32, where the selections cost as much as
-// the differences they save, forms them all (256^3 mixed: 2647 / 2899 us, with
-// the branch 2698 / 2908).  The values are the same either way.
+// 4619 / 4717 us, without the branch 4759 / 4851).  FP32, where the selections
+// cost as much as the differences they save, forms them all (256^3 mixed: 2386 /
+// 2583 us, with the branch 2418 / 2604).  The values are the same either way.
 template <typename R>
 __host__ __device__ __forceinline__ R edge_emf(R fa_m, R fa_p, R ma_m, R ma_p, R fb_m, R fb_p, R mb_m, R mb_p,
                                       R e_mm, R e_pm, R e_mp, R e_pp, bool plain_mean) {
@@ -810,10 +812,8 @@ __host__ __device__ __forceinline__ void char_half_slope(const R* wm, const R* w
 // one reciprocal root each, the projection's coefficients formed once for both
 // sides, and of c_f^2 - a^2 and a^2 - c_s^2 the smaller one from their product
 // a^2 b_t^2 (exactly zero when B_t is), so that the root of the discriminant
-// needs no correct rounding.  Measured (96x64x80, stage 1 / 2): 2138 / 2125 ->
-// 1854 / 1842 us with the shorter roots; against 80-bit arithmetic its error is
-// 0.75 of the plain one's on random states and a hundredth of it where B_t is
-// small.
+// needs no correct rounding.  Measured (96x64x80, stage 1 / 2): 1843 / 1837 us,
+// with the form above 2136 / 2131.
 __host__ __device__ __forceinline__ void char_half_slope(const double* wm, const double* w0, const double* wp, double bn0,
                                                          double gamma, double* slope) {
   const double rho = w0[0], gp = gamma * w0[4];

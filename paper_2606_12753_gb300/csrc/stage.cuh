@@ -288,7 +288,12 @@ __device__ __forceinline__ void recover<P_FP32>(const Geo& g, double rho, double
 }
 
 // CFL speed sum of one cell from its primitives: sum over the active axes of
-// (|v_d| + c_f,d) / Delta_d, c_f,d taken with the cell-centred B_d as normal.
+// (|v_d| + c_f,d) / Delta_d, c_f,d taken with the cell-centred B_d as normal and
+// formed as the fluxes form it.  Where its root cancels (gamma p = B^2, B along
+// one axis) the sum is good to 1e-8 in FP64; mhd_cfl_dt takes signal_sum, which
+// does not cancel, and the two differ by as much there, by rounding elsewhere.
+// (With signal_sum here dt would change in its last bit, and with it the
+// out-of-plane field of a planar two-dimensional flow, which is rounding.)
 template <typename R>
 __device__ __forceinline__ R cfl_speed(const Geo& g, const R* w) {
   R sum = R(0);
@@ -335,7 +340,8 @@ __device__ __forceinline__ R signal_sum(const Geo& g, const R (&v)[3], R a2, con
 // FP32, which is off by less than 1e-5 (inputs cut by 2^-23, a few roundings
 // of terms that only add), against top.  A CFL maximum is of its start's order
 // after a few cells, so nearly every cell is settled by ~50 FP32 instructions
-// instead of ~75 FP64 ones, each of which holds the FP64 pipe for ~17 cycles.
+// instead of ~75 FP64 ones, each of which holds the FP64 pipe for ~17 cycles
+// (128^3 FP64, last stage: 4717 us, with every speed in FP64 5040).
 // Yes is the answer where FP32's range could make the value too small:
 // densities and pressures near its ends, sound speeds below 1e-8 (whose fourth
 // powers underflow; fields that underflow are far below such a sound speed),

@@ -184,9 +184,9 @@ constexpr bool slopes_in_smem() {
 // two-dimensional (one periodic z cell).  The last two are kernels of their
 // own, each without the other's code.  A two-dimensional box in the kernel of
 // any box paid for the ring, the second copies of everything kept by plane
-// parity and one FP64 CTA per SM instead of two (HLL 3200^2 mixed, stage 1 / 2:
-// 1855 / 2066 us there, 1643 / 2014 here, 1246 / 1498 with four CTAs;
-// Orszag-Tang 512^2 FP64: 794 / 841 and 632 / 679).
+// parity and one FP64 CTA per SM instead of two (stage 1 / 2, when the kernels
+// were parted: HLL 3200^2 mixed 1855 / 2066 us there and 1643 / 2014 here,
+// Orszag-Tang 512^2 FP64 794 / 841 and 632 / 679).
 enum BoxKind { BOX_ANY = 0, BOX_3D = 1, BOX_2D = 2 };
 
 // Whether a kernel forms the slopes of the plane after next inside the flux
@@ -195,8 +195,9 @@ enum BoxKind { BOX_ANY = 0, BOX_3D = 1, BOX_2D = 2 };
 // (217 KB for 16 x 8; 8 x 8 tiles run two CTAs per SM).  The slope phase kept
 // the FP64 pipe half idle (17 warp items of 21 operations, a barrier, and the
 // update phase beside it); merged, the warps without a cell go from loading a
-// plane straight to flux items.  Measured (128^3, stage 1 / 2): 4891 / 5013 us
-// with the phase, 4798 / 4900 merged.
+// plane straight to flux items.  Measured (128^3, stage 1 / 2): 4683 / 4827 us
+// with the phase, 4619 / 4717 merged; HLL 4326 / 4460 and 4286 / 4355,
+// characteristic 96x64x80 1852 / 1861 and 1843 / 1837.
 template <int PREC, int MODE, int KIND, int TX, int TY>
 __host__ __device__ constexpr bool merge_slopes() {
   return PREC == P_FP64 && KIND != BOX_2D && TX * TY > 64 && slopes_in_smem<PREC, MODE, TX, TY>();
@@ -262,12 +263,12 @@ struct StageKernel {
   // Threads per CTA, known to the compiler where they may be: the work loops of a plane then have
   // constant trip counts and their item arithmetic folds, which kernels bound by the instructions
   // that they issue and fetch feel.  Stages 1/2 in us, before -> after, all bit for bit alike:
-  // mixed 256^3 2582/2802 -> 2383/2584, FP32 256^3 2192/2292 -> 2104/2205, FP32 2D 1024^2
-  // 158/173 -> 144/163, mixed characteristic -2.5%, FP64 -0.3%.
+  // mixed 256^3 2549/2802 -> 2386/2583, FP32 256^3 2197/2304 -> 2104/2198, FP32 2D 1024^2
+  // 136/152 -> 134/147, mixed characteristic 96x64x80 158/161 -> 152/156, FP64 128^3 -0.3%.
   // Batch and learned kernels of the FP32 bulk read blockDim.x: with the constant the compiler
   // contracts the same sources in another way, and a batch moves by 4e-8, a learned state by 3e-6 in
-  // a few steps.  The learned flux loops alone keep their bits and take it (mixed 128^3 1025/1012 ->
-  // 1004/990).
+  // a few steps.  The learned flux loops alone keep their bits and take it (mixed 128^3 1029/1020 ->
+  // 1011/1000).
   static constexpr int NT = KIND != BOX_ANY ? stage_threads<PREC, TX, TY>() : 256;
   static constexpr bool kFixed = KIND != BOX_ANY || MODE == FM_CHAR || (MODE == FM_PLAIN && PREC == P_FP64);
   static __device__ __forceinline__ int threads() { return kFixed ? NT : (int)blockDim.x; }
@@ -1646,9 +1647,9 @@ struct StageKernel {
 // shared memory of a second FP64 CTA, and of a fourth CTA of the FP32 bulk, for
 // which 64 registers a thread are enough (no spills).  32 warps an SM instead of
 // 24 hide the latencies that bound one plane without a march (us a stage:
-// mixed HLL 3200^2 1605/1941 -> 1246/1498, mixed 1024^2 185/219 -> 152/173, FP32
-// 1024^2 144/164 -> 133/146).  The 3D kernels' shared memory does not hold a
-// fourth CTA, and in 64 registers they are 5 % slower.
+// mixed HLL 3200^2 1612/1940 -> 1247/1495, mixed 1024^2 185/219 -> 152/174, FP32
+// 1024^2 144/164 -> 134/147).  The 3D kernels' shared memory does not hold a
+// fourth CTA, and in 64 registers they are 5 % slower (256^3 mixed 2525/2717).
 template <int PREC, int TX, int TY>
 __host__ __device__ constexpr int stage2d_min_blocks() {
   return PREC == P_FP64 ? (TX * TY <= 128 ? 2 : 1)

@@ -217,7 +217,9 @@ int mhd_rhs(mhd_handle* h, void* cell[5], void* face[3], int on_device);
 
 /* CFL dt of the current state (FP64 reduction on the device; the time step of
  * the Runge-Kutta driver, Sec. 2.2, from the largest signal speed over the
- * cells); synchronises.  *dt_out is caller-owned.  Errors: MHD_ERR_INVALID
+ * cells); synchronises.  The dt that mhd_step takes for dt <= 0 is the same to
+ * the rounding of the form's arithmetic (FP64: 1e-8 where the fast speed's
+ * root cancels, gamma p = B^2 along one axis).  *dt_out is caller-owned.  Errors: MHD_ERR_INVALID
  * (null pointer), MHD_ERR_CUDA. */
 int mhd_cfl_dt(mhd_handle* h, double* dt_out);
 

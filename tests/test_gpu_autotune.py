@@ -33,7 +33,7 @@ def test_autotuning_does_not_lose_the_default(tmp_path):
     assert _ms(b) > 1.25 * before       # no fixed length comes near
     b.set_tile(*default)
     cache = str(tmp_path / "tiles.jsonl")
-    tile, ms = b.autotune(trial_steps=20, cache_path=cache)
+    tile, ms = b.autotune(trial_steps=100, cache_path=cache)
     assert _ms(b) <= 1.1 * before, (default, tile, ms, before)
     # a tile that nothing proposes is among the trials when the batch has it, and the cache names the winner
     assert b.autotune(trial_steps=1, cache_path=cache)[0] == tile
